@@ -9,7 +9,8 @@
 //            output position is the number of smaller columns in the row.
 //  * warp  : one warp per row, a shared hash table (column -> FP64 sum) of 64/256/1024
 //            slots, then the occupied slots are compacted and bitonic-sorted by column.
-//  * block : one block per row, a hash table of 2048 or 8192 slots, compaction, bitonic sort.
+//  * block : one block per row: bitmaps of the row's columns and a rank-indexed array (rows of at
+//            most 2^22 columns), or a hash table of 2048 or 8192 slots, compaction, bitonic sort.
 //  * window: rows with more entries than a block table (k_window.cu).
 // Sums are accumulated with shared-memory FP64 atomics, so their order (and the last bits of
 // a value) can change from run to run; the pattern is always exact.
@@ -207,6 +208,18 @@ __device__ __forceinline__ int hash_claim(int32_t* keys, int32_t key) {
   return -1;
 }
 
+// Adds fa*fb into an FP32 sum sc[0] and its compensation sc[1]: the error-free product fa*fb = ph
+// + pl, and the sum's own rounding error (TwoSum) rebuilt from the value the atomic returns.
+__device__ __forceinline__ void add_compensated(float* sc, float fa, float fb) {
+  const float ph = fa * fb;
+  const float pl = fmaf(fa, fb, -ph);
+  const float old = atomicAdd(&sc[0], ph);
+  const float nw = old + ph;
+  const float bp = nw - old;
+  const float q = (old - (nw - bp)) + (ph - bp);
+  atomicAdd(&sc[1], q + pl);
+}
+
 // Adds the partial product a*b into the slot of `key`. kModeF64: one FP64 atomic. kModeF32C: the
 // slot's 8 bytes hold an FP32 sum and its compensation; the error-free product a*b = ph + pl and
 // the sum's own rounding error (TwoSum, rebuilt from the value the atomic returns) go to the
@@ -220,15 +233,7 @@ __device__ __forceinline__ void hash_accumulate(int32_t* keys, double* vals, int
     return;
   }
   if constexpr (Mode == kModeF32C) {
-    float* sc = reinterpret_cast<float*>(&vals[h]);
-    const float fa = static_cast<float>(a), fb = static_cast<float>(b);
-    const float ph = fa * fb;
-    const float pl = fmaf(fa, fb, -ph);
-    const float old = atomicAdd(&sc[0], ph);
-    const float nw = old + ph;
-    const float bp = nw - old;
-    const float q = (old - (nw - bp)) + (ph - bp);
-    atomicAdd(&sc[1], q + pl);
+    add_compensated(reinterpret_cast<float*>(&vals[h]), static_cast<float>(a), static_cast<float>(b));
   } else {
     atomicAdd(&vals[h], a * b);
   }
@@ -351,6 +356,312 @@ __global__ void __launch_bounds__(256) k_num_warp(DevCsr A, DevCsr B, const int3
   }
 }
 
+// Block rows of a column space of at most kBitmapMaxWidth columns: no hash table and no sort. The
+// row's columns are kept as a bitmap of 32-column words, dense when all the row's words fit `cap`
+// (its table of words), else in two levels: a coarse bit per word of the row, whose prefix count
+// numbers the words that hold a column (at most one per entry of C, so they fit the table). The
+// prefix count over the words gives every column its rank, the products are added into a
+// rank-indexed array and the row leaves in rank order.
+//
+// A row whose products fit the block's registers (kHeld per thread, one chunk of A entries) reads
+// B once: its columns and products stay in registers between the marking and the accumulation.
+// Longer rows enumerate their products in each pass.
+//
+// Bound by the latency of the gathers and the barriers between the passes. 256 threads with 64
+// registers, so that four rows are in flight on an SM; the hash table and bitonic sort of
+// k_num_block are bound by the sort's shared-memory traffic instead. Both block classes, hash
+// and bitonic sort -> bitmaps: 20,000^2 uniform (19,400 rows of 1,540 entries) 3.83 -> 0.36 ms,
+// R-MAT 2^17 2.67 -> 0.46 ms, R-MAT 2^19 7.87 -> 1.19 ms.
+constexpr int kHeld = 8;   // products per thread held in registers
+constexpr int kStep = 4;   // products per thread in one step (loads in flight)
+constexpr int64_t kBitmapMaxWidth = int64_t(1) << 22;   // coarse words: 16 KB
+
+// Coarse words a block keeps: none when every row's words fit the table of `cap` words.
+__host__ __device__ inline int bitmap_coarse_words(int64_t width, int cap) {
+  const int64_t words = (width + 31) >> 5;
+  return words <= cap ? 0 : static_cast<int>((words + 31) >> 5);
+}
+
+template <int NT>
+struct BitmapChunk {
+  int64_t bs[NT];        // per non-empty B row of the chunk: its start in B,
+  double av[NT];         //   a_ik,
+  int32_t excl[NT + 1];  //   its first product's number (and the total last)
+  long long scan64[33];
+  int32_t scan[33];
+  int32_t ctl[2];        // segments, products
+};
+
+// The A entries [base, base + NT) of the row, their non-empty B rows compacted into ck.
+template <int NT, int Mode>
+__device__ __forceinline__ void bitmap_chunk(const DevCsr& A, const DevCsr& B, int64_t a0, int64_t na, int64_t base,
+                                             BitmapChunk<NT>& ck) {
+  const int64_t e = base + threadIdx.x;
+  int64_t bs = 0;
+  int32_t len = 0;
+  double av = 0.0;
+  if (e < na) {
+    const int32_t k = A.col[a0 + e];
+    av = value_at<Mode>(A.val, a0 + e);
+    bs = B.rp[k];
+    len = static_cast<int32_t>(B.rp[k + 1] - bs);
+  }
+  const long long packed = (static_cast<long long>(len > 0) << 32) | static_cast<long long>(len);
+  long long tot;
+  const long long ex = block_excl_scan<long long>(packed, ck.scan64, &tot);
+  if (len > 0) {
+    const int pos = static_cast<int>(ex >> 32);
+    ck.bs[pos] = bs;
+    ck.av[pos] = av;
+    ck.excl[pos] = static_cast<int32_t>(ex & 0xffffffffLL);
+  }
+  if (threadIdx.x == 0) {
+    ck.ctl[0] = static_cast<int32_t>(tot >> 32);
+    ck.ctl[1] = static_cast<int32_t>(tot & 0xffffffffLL);
+    ck.excl[ck.ctl[0]] = ck.ctl[1];
+  }
+  __syncthreads();
+}
+
+// The chunk's products, one contiguous range per warp, kStep groups of 32 per call: f(q, j, av)
+// with kStep indices into B (-1: none) and their a_ik, q the call's number (of a chunk that fits the
+// registers: below kHeld / kStep, and known at compile time; else 0).
+template <int NT, typename F>
+__device__ __forceinline__ void bitmap_for_each(const BitmapChunk<NT>& ck, bool fits, F&& f) {
+  const int wid = threadIdx.x >> 5;
+  const int nent = ck.ctl[0];
+  const int32_t total = ck.ctl[1];
+  int32_t per = (total + NT / 32 - 1) / (NT / 32);
+  per = (per + 31) & ~31;
+  const int32_t lo = wid * per;
+  const int32_t hi = total < lo + per ? total : lo + per;
+  if (lo >= hi) return;
+  auto walk = make_walker<double>(ck.excl, ck.bs, nent, search_owner(ck.excl, nent, lo),
+                                  [&](int sgm) { return ck.av[sgm]; });
+  int64_t j[kStep];
+  double av[kStep];
+  if (fits) {
+#pragma unroll
+    for (int q = 0; q < kHeld / kStep; ++q) {
+      const int32_t p0 = lo + q * 32 * kStep;
+      if (p0 < hi) {
+        walk.template step_many<kStep>(p0, hi, j, av);
+        f(q, j, av);
+      }
+    }
+  } else {
+    for (int32_t p0 = lo; p0 < hi; p0 += 32 * kStep) {
+      walk.template step_many<kStep>(p0, hi, j, av);
+      f(0, j, av);
+    }
+  }
+}
+
+// pre[w] = bits set in words[0, w); returns the number of bits set in words[0, n). Each thread
+// takes a run of consecutive words. Ends with a barrier.
+template <int NT>
+__device__ __forceinline__ int bitmap_prefix(const uint32_t* words, uint16_t* pre, int n, int32_t* scan) {
+  const int k = (n + NT - 1) / NT;
+  const int lo = min(n, static_cast<int>(threadIdx.x) * k), hi = min(n, lo + k);
+  int c = 0;
+  for (int w = lo; w < hi; ++w) c += __popc(words[w]);
+  int32_t total;
+  int run = block_excl_scan<int32_t>(c, scan, &total);
+  for (int w = lo; w < hi; ++w) {
+    pre[w] = static_cast<uint16_t>(min(run, 65535));
+    run += __popc(words[w]);
+  }
+  __syncthreads();
+  return total;
+}
+
+// One partial product in eight bytes: a*b (kModeF64) or the FP32 pair (a, b) (kModeF32C).
+template <int Mode>
+__device__ __forceinline__ double held_product(double a, double b) {
+  if constexpr (Mode == kModeF32C) {
+    const float2 ab = make_float2(static_cast<float>(a), static_cast<float>(b));
+    return *reinterpret_cast<const double*>(&ab);
+  } else {
+    return a * b;
+  }
+}
+
+// Adds a held product into an eight-byte slot (the modes of hash_accumulate).
+template <int Mode>
+__device__ __forceinline__ void add_held(double* slot, double held) {
+  if constexpr (Mode == kModeF32C) {
+    const float2 ab = *reinterpret_cast<const float2*>(&held);
+    add_compensated(reinterpret_cast<float*>(slot), ab.x, ab.y);
+  } else {
+    atomicAdd(slot, held);
+  }
+}
+
+template <int NT, int Mode>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
+                                                     int64_t count, const int64_t* __restrict__ c_off,
+                                                     int32_t* __restrict__ ccol, void* __restrict__ cval,
+                                                     const int32_t* __restrict__ abase,
+                                                     const int32_t* __restrict__ awidth, int64_t width_all, int cap,
+                                                     int32_t* __restrict__ row_flag,
+                                                     const int32_t* __restrict__ negflag, uint32_t* err) {
+  extern __shared__ double smem_f64[];
+  __shared__ BitmapChunk<NT> ck;
+  double* vals = smem_f64;                                          // [cap], by rank
+  int32_t* colbuf = reinterpret_cast<int32_t*>(vals + cap);         // [cap], the row's columns by rank
+  int32_t* gword = colbuf + cap;                                    // [cap], two levels: word number of a table word
+  uint32_t* fine = reinterpret_cast<uint32_t*>(gword + cap);        // [cap], the word table (zero between rows)
+  uint32_t* coarse = fine + cap;                                    // a bit per word (zero between rows)
+  const int coarse_all = bitmap_coarse_words(width_all, cap);
+  uint16_t* fpre = reinterpret_cast<uint16_t*>(coarse + coarse_all);   // [cap]
+  uint16_t* cpre = fpre + cap;                                         // [coarse_all]
+  for (int t = threadIdx.x; t < cap + coarse_all; t += NT) fine[t] = 0u;
+  for (int64_t r = blockIdx.x; r < count; r += gridDim.x) {
+    const int32_t i = perm[r];
+    const int64_t a0 = A.rp[i];
+    const int64_t na = A.rp[i + 1] - a0;
+    const int64_t off = c_off[i];
+    const int64_t len = c_off[i + 1] - off;
+    const int32_t cb = abase ? abase[i] : 0;   // the row's columns are [cb, cb + width)
+    const uint32_t width = static_cast<uint32_t>(awidth ? awidth[i] : width_all);
+    const int words = static_cast<int>((width + 31) >> 5);
+    const bool direct = words <= cap;
+    if (Mode == kModeF32C && threadIdx.x == 0 && !f32c_hash_row_ok(negflag, na)) row_flag[i] = 1;
+    __syncthreads();   // the previous row's clearing of the bitmaps
+    // the table word of column rel (two levels), -1 past the table (a row counted otherwise)
+    auto table_word = [&](uint32_t rel) {
+      const uint32_t cw = coarse[rel >> 10];
+      const int g = cpre[rel >> 10] + __popc(cw & ((1u << ((rel >> 5) & 31)) - 1u));
+      return g < cap ? g : -1;
+    };
+    // held: per product of the step its table word * 32 + bit, -1 for none; of a held row only
+    int32_t held[kHeld];
+    double pv[kHeld];
+    bool bad = false, keep = false;
+    // pass 1: the words (one level) or the coarse bits of the row's columns
+    for (int64_t base = 0; base < na; base += NT) {
+      bitmap_chunk<NT, Mode>(A, B, a0, na, base, ck);
+      keep = na <= NT && ck.ctl[1] <= NT * kHeld;
+#pragma unroll
+      for (int u = 0; u < kHeld; ++u) held[u] = -1;
+      bitmap_for_each<NT>(ck, keep, [&](int q, const int64_t (&j)[kStep], const double (&av)[kStep]) {
+        int32_t c[kStep];
+#pragma unroll
+        for (int u = 0; u < kStep; ++u) c[u] = j[u] >= 0 ? B.col[j[u]] : 0;
+        if (keep) {
+#pragma unroll
+          for (int u = 0; u < kStep; ++u)
+            pv[q * kStep + u] = j[u] >= 0 ? held_product<Mode>(av[u], value_at<Mode>(B.val, j[u])) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kStep; ++u) {
+          if (j[u] < 0) continue;
+          const uint32_t rel = static_cast<uint32_t>(c[u] - cb);
+          if (rel >= width) { bad = true; continue; }
+          if (direct) atomicOr(&fine[rel >> 5], 1u << (rel & 31));
+          else atomicOr(&coarse[rel >> 10], 1u << ((rel >> 5) & 31));
+          held[q * kStep + u] = static_cast<int32_t>(rel);
+        }
+      });
+      __syncthreads();
+    }
+    int nwords = words;
+    const int cwords = (words + 31) >> 5;
+    if (!direct) {
+      const int groups = bitmap_prefix<NT>(coarse, cpre, cwords, ck.scan);
+      nwords = groups < cap ? groups : cap;
+      for (int w = threadIdx.x; w < cwords; w += NT) {
+        int g = cpre[w];
+        for (uint32_t m = coarse[w]; m; m &= m - 1, ++g)
+          if (g < cap) gword[g] = w * 32 + __ffs(m) - 1;
+      }
+      // pass 2: the table words
+      if (keep) {
+#pragma unroll
+        for (int u = 0; u < kHeld; ++u) {
+          if (held[u] < 0) continue;
+          const int g = table_word(held[u]);
+          const int bit = held[u] & 31;
+          if (g >= 0) atomicOr(&fine[g], 1u << bit);
+          held[u] = g >= 0 ? g * 32 + bit : -1;
+        }
+      } else {
+        for (int64_t base = 0; base < na; base += NT) {
+          bitmap_chunk<NT, Mode>(A, B, a0, na, base, ck);
+          bitmap_for_each<NT>(ck, false, [&](int, const int64_t (&j)[kStep], const double (&)[kStep]) {
+            int32_t c[kStep];
+#pragma unroll
+            for (int u = 0; u < kStep; ++u) c[u] = j[u] >= 0 ? B.col[j[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < kStep; ++u) {
+              const uint32_t rel = static_cast<uint32_t>(c[u] - cb);
+              if (j[u] < 0 || rel >= width) continue;
+              const int g = table_word(rel);
+              if (g >= 0) atomicOr(&fine[g], 1u << (rel & 31));
+            }
+          });
+          __syncthreads();
+        }
+      }
+      __syncthreads();
+    }
+    const int cnt = bitmap_prefix<NT>(fine, fpre, nwords, ck.scan);
+    const int n_out = cnt < len ? min(cnt, cap) : static_cast<int>(min(len, static_cast<int64_t>(cap)));
+    if (cnt != len) bad = true;
+    for (int t = threadIdx.x; t < n_out; t += NT) vals[t] = 0.0;
+    __syncthreads();
+    // pass 3: the products by rank
+    auto add = [&](int g, int bit, double p) {
+      const int rk = fpre[g] + __popc(fine[g] & ((1u << bit) - 1u));
+      if (rk < n_out) add_held<Mode>(&vals[rk], p);
+    };
+    if (keep) {
+#pragma unroll
+      for (int u = 0; u < kHeld; ++u)
+        if (held[u] >= 0) add(held[u] >> 5, held[u] & 31, pv[u]);
+      __syncthreads();
+    } else {
+      for (int64_t base = 0; base < na; base += NT) {
+        bitmap_chunk<NT, Mode>(A, B, a0, na, base, ck);
+        bitmap_for_each<NT>(ck, false, [&](int, const int64_t (&j)[kStep], const double (&av)[kStep]) {
+          int32_t c[kStep];
+          double p[kStep];
+#pragma unroll
+          for (int u = 0; u < kStep; ++u) {
+            c[u] = j[u] >= 0 ? B.col[j[u]] : 0;
+            p[u] = j[u] >= 0 ? held_product<Mode>(av[u], value_at<Mode>(B.val, j[u])) : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < kStep; ++u) {
+            const uint32_t rel = static_cast<uint32_t>(c[u] - cb);
+            if (j[u] < 0 || rel >= width) continue;
+            const int g = direct ? static_cast<int>(rel >> 5) : table_word(rel);
+            if (g >= 0) add(g, rel & 31, p[u]);
+          }
+        });
+        __syncthreads();
+      }
+    }
+    // the columns by rank, and the bitmaps cleared for the next row
+    for (int w = threadIdx.x; w < nwords; w += NT) {
+      uint32_t m = fine[w];
+      if (!m) continue;
+      const int col0 = 32 * (direct ? w : gword[w]);
+      for (int rk = fpre[w]; m; m &= m - 1, ++rk)
+        if (rk < n_out) colbuf[rk] = col0 + __ffs(m) - 1;
+      fine[w] = 0u;
+    }
+    if (!direct)
+      for (int w = threadIdx.x; w < cwords; w += NT) coarse[w] = 0u;
+    __syncthreads();
+    for (int t = threadIdx.x; t < n_out; t += NT) {
+      ccol[off + t] = colbuf[t];
+      store_value<Mode>(cval, off + t, vals[t]);
+    }
+    if (bad) set_error(err, kErrCount);
+  }
+}
+
 template <int LOG2S, int NT, int Mode>
 __global__ void __launch_bounds__(NT) k_num_block(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
                                                   int64_t count, const int64_t* __restrict__ c_off,
@@ -453,11 +764,25 @@ int launch_num_warp(int log2S, int mode, const DevCsr& A, const DevCsr& B, const
 }
 
 int launch_num_block(int log2S, int mode, const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
-                     const int64_t* c_off, int32_t* ccol, void* cval, const int32_t* abase, int32_t* row_flag,
-                     const int32_t* negflag, uint32_t* err, int num_sms, cudaStream_t s) {
+                     const int64_t* c_off, int32_t* ccol, void* cval, const int32_t* abase, const int32_t* awidth,
+                     int64_t width, int max_nnz, int32_t* row_flag, const int32_t* negflag, uint32_t* err,
+                     int num_sms, cudaStream_t s) {
   if (count <= 0) return 0;
-  const size_t sm = (size_t(1) << log2S) * 12;
   const bool f32c = mode == kModeF32C;
+  // the coarse bitmap of wider rows would not leave room for four rows on an SM: they hash
+  if (width <= kBitmapMaxWidth) {
+    const int cap = log2S == 11 ? 1024 : (max_nnz <= 2048 ? 2048 : 4096);
+    const int cw = bitmap_coarse_words(width, cap);
+    const size_t sm = size_t(cap) * (8 + 4 + 4 + 4 + 2) + size_t(cw) * 6;
+    auto go = [&](auto kernel) {
+      if (sm > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+      kernel<<<grid_rows(count, 1, num_sms * 16), 256, sm, s>>>(A, B, perm, count, c_off, ccol, cval, abase, awidth, width,
+                                                               cap, row_flag, negflag, err);
+    };
+    f32c ? go(k_num_bitmap<256, kModeF32C>) : go(k_num_bitmap<256, kModeF64>);
+    return 1;
+  }
+  const size_t sm = (size_t(1) << log2S) * 12;
   auto go = [&](auto kernel, int nt, int per_sm) {
     if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
     kernel<<<grid_rows(count, 1, num_sms * per_sm), nt, sm, s>>>(A, B, perm, count, c_off, ccol, cval, abase, row_flag,

@@ -635,9 +635,9 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
       const int32_t* neg = f32c ? p->counters + 8 : nullptr;
       stage_begin(p, SPGEMM_STAGE_NUM_BLOCK, s);
       nl = launch_num_block(13, mode, p->A, p->B, seg(kNumBlock2), cnt(kNumBlock2), p->c_off, C->col, C->val,
-                            p->abase, flag, neg, err, p->num_sms, s);
+                            p->abase, p->awidth, p->width, p->cp.block_max, flag, neg, err, p->num_sms, s);
       nl += launch_num_block(11, mode, p->A, p->B, seg(kNumBlock1), cnt(kNumBlock1), p->c_off, C->col, C->val,
-                             p->abase, flag, neg, err, p->num_sms, s);
+                             p->abase, p->awidth, p->width, p->cp.block_max, flag, neg, err, p->num_sms, s);
       stage_end(p, SPGEMM_STAGE_NUM_BLOCK, nl, s);
       stage_begin(p, SPGEMM_STAGE_NUM_WARP, s);
       nl = launch_num_warp(10, mode, p->A, p->B, seg(kNumWarp3), cnt(kNumWarp3), p->c_off, C->col, C->val, p->abase,
