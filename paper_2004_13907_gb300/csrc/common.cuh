@@ -110,6 +110,11 @@ constexpr int kBlockShift = 12;
 constexpr int kBlockCols = 1 << kBlockShift;   // columns per block, 4096
 constexpr int kBlockWords = kBlockCols / 32;   // bitmap words per block
 constexpr int kSymWinBits = 1 << 20;           // symbolic bitmap window (128 KB)
+// A plan whose windowed rows all have a stored bitmap counts them in sub-blocks instead
+// (k_winteam.cu): small enough that a warp's window holds any of them.
+constexpr int kSubShift = 10;
+constexpr int kSubCols = 1 << kSubShift;
+constexpr int kMaxSub = kSymWinBits / kSubCols;
 constexpr int kSymWinThreads = 1024;           // threads of the windowed symbolic kernel
 
 __device__ __forceinline__ void set_error(uint32_t* err, uint32_t code) { atomicOr(err, code); }

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kSymWinThreads, 1) k_sym_window(DevCsr A, DevC
                                                                int32_t* __restrict__ nnz_row,
                                                                int32_t* __restrict__ win_slot,
                                                                uint16_t* __restrict__ blockcnt,
-                                                               int64_t nblocks, int32_t* cursor,
+                                                               int64_t nblocks, int sub, int32_t* cursor,
                                                                const int32_t* __restrict__ abase,
                                                                const int32_t* __restrict__ awidth,
                                                                int64_t width_all, uint32_t* __restrict__ wbits,
@@ -293,9 +293,16 @@ __global__ void __launch_bounds__(kSymWinThreads, 1) k_sym_window(DevCsr A, DevC
         uint4* p = reinterpret_cast<uint4*>(bm + (b * kBlockWords - (r0 >> 5))) + lane;
         const uint4 v = *p;
         int c = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
-        c = warp_sum(c);
+        // 8 lanes hold a sub-block
+        constexpr int kSubLanes = kSubCols / 128;
+#pragma unroll
+        for (int d = 1; d < kSubLanes; d <<= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
+        const int64_t sb = b * (kBlockCols / kSubCols) + lane / kSubLanes;
+        if (sub && lane % kSubLanes == 0 && sb < nblocks) cnts[sb] = static_cast<uint16_t>(c);
+#pragma unroll
+        for (int d = kSubLanes; d < 32; d <<= 1) c += __shfl_xor_sync(0xffffffffu, c, d);
         if (lane == 0) {
-          cnts[b] = static_cast<uint16_t>(c);
+          if (!sub) cnts[b] = static_cast<uint16_t>(c);
           if (c) atomicAdd(&s_total, static_cast<unsigned long long>(c));
         }
         // a stored row has one window, starting at block 0
@@ -366,7 +373,7 @@ int launch_sym_block(int log2S, const DevCsr& A, const DevCsr& B, const int32_t*
 
 int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
                        int32_t* counter, int32_t* nnz_row, int32_t* win_slot, uint16_t* blockcnt,
-                       int64_t nblocks, int32_t* cursor, const int32_t* abase, const int32_t* awidth,
+                       int64_t nblocks, int sub, int32_t* cursor, const int32_t* abase, const int32_t* awidth,
                        int64_t width, uint32_t* wbits, int64_t wcap, unsigned long long* wcur, int64_t* woff,
                        int num_sms, uint32_t* err, cudaStream_t s) {
   if (count <= 0) return 0;
@@ -375,7 +382,7 @@ int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
   const int64_t g = count < num_sms ? count : num_sms;
   k_sym_window<<<static_cast<unsigned>(g), kSymWinThreads, sm, s>>>(A, B, perm, count, counter, nnz_row,
-                                                                 win_slot, blockcnt, nblocks, cursor,
+                                                                 win_slot, blockcnt, nblocks, sub, cursor,
                                                                  abase, awidth, width, wbits, wcap, wcur, woff, err);
   return 1;
 }

@@ -115,10 +115,10 @@ int launch_sym_block(int log2S, const DevCsr& A, const DevCsr& B, const int32_t*
 // (the block-count stride of a row) covers the widest row. wbits (may be NULL) receives, for each
 // row no wider than one symbolic window, its column bitmap (128 words per block of the row) at
 // word woff[slot], reserved from the cursor *wcur; -1 when the wcap words are used up or the row
-// is wider.
+// is wider. sub: blockcnt counts sub-blocks of kSubCols columns (nblocks their number).
 int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
                        int32_t* counter, int32_t* nnz_row, int32_t* win_slot, uint16_t* blockcnt,
-                       int64_t nblocks, int32_t* cursor, const int32_t* abase, const int32_t* awidth,
+                       int64_t nblocks, int sub, int32_t* cursor, const int32_t* abase, const int32_t* awidth,
                        int64_t width, uint32_t* wbits, int64_t wcap, unsigned long long* wcur, int64_t* woff,
                        int num_sms, uint32_t* err, cudaStream_t s);
 
@@ -153,6 +153,19 @@ int64_t rerun_group_rows(int64_t width, int64_t budget_bytes);
 int launch_rerun_dense(const DevCsr& A, const DevCsr& B, const int32_t* rows, int64_t nrows, const int64_t* c_off,
                        int32_t* ccol, float* cval, const int32_t* abase, int64_t width, double* dense,
                        int64_t group_rows, int num_sms, uint32_t* err, cudaStream_t s);
+
+// ---- windowed rows of plans that store all their bitmaps (k_winteam.cu). The list of windows (its
+// bytes, and room for *cap windows; their number at *n_wins), built once per plan; the split table of
+// B by sub-blocks (B.rows * nsub + 1 words); the numeric pass itself, columns included.
+int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merge_cap, int64_t* cap);
+int launch_win_plan(const DevCsr& A, const int32_t* perm, int64_t count, const int32_t* win_slot, int64_t nslots,
+                    const uint16_t* subcnt, int64_t nsub, int32_t merge_cap, const int64_t* c_off, const int64_t* woff,
+                    const int32_t* abase, const int32_t* awidth, int64_t width, void* wins, int64_t cap,
+                    int32_t* n_wins, int num_sms, uint32_t* err, cudaStream_t s);
+int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint32_t* split, cudaStream_t s);
+int launch_num_winteam(const DevCsr& A, const DevCsr& B, const void* wins, const int32_t* n_wins, int64_t wins_cap,
+                       int32_t* counter, const uint16_t* subcnt, int64_t nsub, const uint32_t* split, int32_t* ccol,
+                       double* cval, const uint32_t* wbits, int num_sms, uint32_t* err, cudaStream_t s);
 
 int64_t split_table_bytes(int64_t brows, int64_t nblocks);
 int launch_bsplit(const DevCsr& B, int64_t nblocks, const int32_t* bbase, int32_t* split, cudaStream_t s);

@@ -342,15 +342,20 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
     const int64_t cnt_bytes = nwin * p->nblocks * 2;
     if (cnt_bytes > (int64_t(8) << 30))
       return set_error_msg(SPGEMM_ERR_UNSUPPORTED, "windowed rows need %lld bytes of block counts", (long long)cnt_bytes);
-    p->blockcnt = ws_get<uint16_t>(p, nwin * p->nblocks, &st);
-    p->win_slot = ws_get<int32_t>(p, m, &st);
-    p->cursor = ws_get<int32_t>(p, A->nnz, &st);
-    if (st) return st;
     // room for the windowed rows' column bitmaps (one 128-word block per 4096 columns of the row),
     // within the budget; rows that find it full keep the marking pass in the numeric kernel
     const int64_t budget = (int64_t(p->opts.window_cols_max_mb > 0 ? p->opts.window_cols_max_mb : 0) << 20) / 4;
     const int64_t need = nwin * p->nblocks * kBlockWords;
     p->wcap = need < budget ? need : budget;
+    // all of them stored: the warp-per-window numeric pass, which plans by sub-blocks and numbers
+    // B's entries with 32 bits
+    p->sub = p->prec == SPGEMM_F64 && p->opts.fp64_accumulate == 0 && need <= budget && p->width <= kSymWinBits &&
+             B->nnz <= 0x7fffffffLL;
+    if (p->sub) p->nblocks = (p->width + kSubCols - 1) / kSubCols;
+    p->blockcnt = ws_get<uint16_t>(p, nwin * p->nblocks, &st);
+    p->win_slot = ws_get<int32_t>(p, m, &st);
+    p->cursor = ws_get<int32_t>(p, A->nnz, &st);
+    if (st) return st;
     if (p->wcap > 0) {
       p->wbits = ws_get<uint32_t>(p, p->wcap, &st);
       p->wcur = ws_get<unsigned long long>(p, 1, &st);
@@ -417,7 +422,7 @@ spgemm_status symbolic_run(spgemm_plan_s* p, cudaStream_t s) {
     stage_begin(p, SPGEMM_STAGE_SYM_WINDOW, s);
     if (p->wcur) cudaMemsetAsync(p->wcur, 0, sizeof(unsigned long long), s);
     nl = launch_sym_window(p->A, p->B, seg(kSymWin0), p->sym_off[kSymWin3 + 1] - p->sym_off[kSymWin0],
-                           p->counters + 0, p->nnz_row, p->win_slot, p->blockcnt, p->nblocks, p->cursor,
+                           p->counters + 0, p->nnz_row, p->win_slot, p->blockcnt, p->nblocks, p->sub, p->cursor,
                            p->abase, p->awidth, p->width, p->wbits, p->wcap, p->wcur, p->woff, p->num_sms, err,
                            s);
     stage_end(p, SPGEMM_STAGE_SYM_WINDOW, nl, s);
@@ -476,7 +481,8 @@ void plan_bytes_bounds(int64_t m, int64_t a_nnz, int64_t width, int a_rowptr32, 
   const int64_t stored = stored_words > 0 ? ws_rounded(4 * (row_words < stored_words ? row_words : stored_words)) +
                                                 ws_rounded(8) + ws_rounded(8 * m)
                                           : 0;
-  const int64_t window = ws_rounded(2 * m * nblocks) + ws_rounded(4 * m) + ws_rounded(4 * a_nnz) + stored;
+  const int64_t counted = wbits_mb > 0 && width <= kSymWinBits ? (width + kSubCols - 1) / kSubCols : nblocks;
+  const int64_t window = ws_rounded(2 * m * counted) + ws_rounded(4 * m) + ws_rounded(4 * a_nnz) + stored;
   *lo = fixed;
   *hi = fixed + tiles + window;
 }
@@ -499,6 +505,42 @@ int64_t window_list_cap(const spgemm_plan_s* p, int64_t nwin) {
   return cap < kListCapMax ? cap : kListCapMax;
 }
 
+int64_t window_list_bytes(const spgemm_plan_s* p, int64_t nwin, int64_t* cap) {
+  unsigned long long entries = 0;
+  for (int c = kNumWin0; c <= kNumWin3; ++c) entries += p->cls_sums[c][2];
+  return win_list_bytes(nwin, static_cast<int64_t>(entries), p->nblocks, p->opts.window_hash_fill, cap);
+}
+
+int64_t split_sub_bytes(const spgemm_plan_s* p) { return p->B.rows * p->nblocks * int64_t(sizeof(uint32_t)); }
+
+// The windowed rows of a plan whose windowed rows all have a stored bitmap (p->sub). Returns the
+// launches made, or -1 when a workspace could not be allocated.
+int numeric_windows(spgemm_plan_s* p, const int32_t* perm, int64_t nwin, int64_t nslots, spgemm_csr_out* C,
+                    cudaStream_t s) {
+  if (nwin <= 0) return 0;
+  int nl = 0;
+  if (!p->split_tried) {
+    // split table of B, once per plan, when it fits the budget (else the kernel searches)
+    p->split_tried = true;
+    const int64_t bytes = split_sub_bytes(p);
+    if (bytes <= (int64_t(p->opts.window_split_max_mb) << 20)) {
+      p->split_sub = static_cast<uint32_t*>(p->ws.get(static_cast<size_t>(bytes) + sizeof(uint32_t)));
+      if (p->split_sub) nl += launch_bsplit_sub(p->B, p->nblocks, p->bbase, p->split_sub, s);
+    }
+  }
+  if (!p->wins) {
+    const int64_t bytes = window_list_bytes(p, nwin, &p->wins_cap);
+    p->wins = p->ws.get(static_cast<size_t>(bytes));
+    if (!p->wins) return -1;
+    nl += launch_win_plan(p->A, perm, nwin, p->win_slot, nslots, p->blockcnt, p->nblocks, p->opts.window_hash_fill,
+                          p->c_off, p->woff, p->abase, p->awidth, p->width, p->wins, p->wins_cap, p->counters + 9,
+                          p->num_sms, &p->summary->err, s);
+  }
+  return nl + launch_num_winteam(p->A, p->B, p->wins, p->counters + 9, p->wins_cap, p->counters + 1, p->blockcnt,
+                                 p->nblocks, p->split_sub, C->col, static_cast<double*>(C->val), p->wbits, p->num_sms,
+                                 &p->summary->err, s);
+}
+
 }  // namespace
 
 int64_t numeric_extra_bytes(const spgemm_plan_s* p) {
@@ -515,7 +557,12 @@ int64_t numeric_extra_bytes(const spgemm_plan_s* p) {
     if (!p->rerun_flag) extra += 2 * ws_rounded(4 * m);   // flags and list of FP64 reruns
     if (!p->bexp) extra += ws_rounded(2 * p->B.rows);     // exponent bound per row of B
   }
-  if (nwin > 0 && !p->split_tried) {
+  if (p->sub && nwin > 0) {
+    if (!p->split_tried && split_sub_bytes(p) <= (int64_t(p->opts.window_split_max_mb) << 20))
+      extra += ws_rounded(split_sub_bytes(p) + 4);
+    int64_t cap = 0;
+    if (!p->wins) extra += ws_rounded(window_list_bytes(p, nwin, &cap));
+  } else if (nwin > 0 && !p->split_tried) {
     const int64_t bytes = split_table_bytes(p->B.rows, p->nblocks);
     if (bytes <= (int64_t(p->opts.window_split_max_mb) << 20)) {
       extra += ws_rounded(bytes);
@@ -589,7 +636,12 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
     // error bound needs no sum of |p|), read by the window kernel on the device
     if (f32c && nwh > 0) nl += launch_negative_check(p->A.val, p->A.nnz, p->B.val, p->B.nnz, p->counters + 8,
                                                      p->num_sms, s);
-    if (nwin > 0 && !p->split_tried) {
+    if (p->sub) {
+      const int n = numeric_windows(p, seg(kNumWin0), nwin, nslots, C, s);
+      if (n < 0) return set_error_msg(SPGEMM_ERR_OOM, "device workspace allocation of the window list failed");
+      nl += n;
+    }
+    if (!p->sub && nwin > 0 && !p->split_tried) {
       // split table of B, once per plan, when it fits the budget (else the kernel searches)
       p->split_tried = true;
       const int64_t bytes = split_table_bytes(p->B.rows, p->nblocks);
@@ -598,7 +650,7 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
         if (p->split) nl += launch_bsplit(p->B, p->nblocks, p->bbase, p->split, s);
       }
     }
-    if (nwin > 0 && !p->lists_tried && !fx) {
+    if (!p->sub && nwin > 0 && !p->lists_tried && !fx) {
       p->lists_tried = true;
       const int64_t cap = p->split ? window_list_cap(p, nwin) : 0;
       const int64_t n = num_window_blocks(nwin, p->num_sms) * cap;
@@ -609,7 +661,8 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
         if (p->list_bs && p->list_len && p->list_av) p->list_cap = cap;
       }
     }
-    nl += launch_num_window(fx ? kModeF64X : mode, p->A, p->B, seg(kNumWin0), nwin, p->counters + 1, p->c_off,
+    if (!p->sub)
+      nl += launch_num_window(fx ? kModeF64X : mode, p->A, p->B, seg(kNumWin0), nwin, p->counters + 1, p->c_off,
                             p->win_slot, p->blockcnt, p->nblocks, nslots, p->split, p->opts.window_hash_fill, C->col,
                             C->val, p->rerun_flag, p->abase, p->awidth, p->width, p->wbits, p->woff, p->bexp,
                             nullptr, f32c ? p->counters + 8 : nullptr, fx ? nullptr : p->list_bs,
@@ -627,7 +680,7 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
     }
     stage_end(p, SPGEMM_STAGE_NUM_WINDOW, nl, s);
     stage_begin(p, SPGEMM_STAGE_NUM_EXPAND, s);
-    nl = launch_expand_cols(seg(kNumWin0), nwin, p->win_slot, p->woff, p->wbits, p->blockcnt, p->nblocks, p->c_off,
+    nl = p->sub ? 0 : launch_expand_cols(seg(kNumWin0), nwin, p->win_slot, p->woff, p->wbits, p->blockcnt, p->nblocks, p->c_off,
                             p->awidth, p->width, C->col, p->num_sms, err, s);
     stage_end(p, SPGEMM_STAGE_NUM_EXPAND, nl, s);
     {

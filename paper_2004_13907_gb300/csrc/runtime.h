@@ -53,7 +53,11 @@ struct spgemm_plan_s {
   int32_t* counters = nullptr;       // device, 16 ints
   int32_t* win_slot = nullptr;
   uint16_t* blockcnt = nullptr;
-  int64_t nblocks = 0;
+  int64_t nblocks = 0;               // column blocks, or sub-blocks (sub), of the widest row
+  bool sub = false;                  // every windowed row has a stored bitmap: the pass over a list of windows
+  uint32_t* split_sub = nullptr;     // sub: split table of B by sub-blocks
+  void* wins = nullptr;              // sub: the list of windows (counters[9] of them)
+  int64_t wins_cap = 0;
   int32_t* cursor = nullptr;
   int32_t* split = nullptr;          // column-block split table of B (windowed numeric rows)
   uint32_t* wbits = nullptr;         // column bitmaps of windowed rows, stored by the symbolic pass
