@@ -312,7 +312,7 @@ void batch_prepare_bounds(int64_t n_jobs, const spgemm_csr_in* A, const spgemm_c
                           ws_rounded(8 * (inner + 1)) + ws_rounded(4 * b_nnz) + ws_rounded(vb * b_nnz) +
                           ws_rounded(4 * inner) + ws_rounded(4);
   int64_t plo = 0, phi = 0;
-  plan_bytes_bounds(rows, a_nnz, width, 0, 0, inner, b_nnz, opts->validate, opts->window_cols_max_mb, &plo, &phi);
+  plan_bytes_bounds(rows, a_nnz, width, 0, 0, inner, opts->window_cols_max_mb, &plo, &phi);
   *lo = stacked + plo;
   *hi = stacked + phi;
 }

@@ -18,6 +18,14 @@ struct DevCsr {
   const void* val;
 };
 
+// A CSR pattern with its row pointers as the caller stores them.
+struct CsrArrays {
+  int64_t rows, cols, nnz;
+  const void* rp;        // int32 or int64 row pointers
+  int32_t rp64;
+  const int32_t* col;
+};
+
 // Summary the host reads back after the plan and after the symbolic pass.
 struct Summary {
   int64_t class_off[kMaxClasses + 1];
@@ -82,11 +90,14 @@ int launch_fetch(const void* src, void* dst, int64_t bytes, cudaStream_t s);
 // out[t] = in[r0 + t] - base for t < n1 (in: int32 or int64 row pointers).
 int launch_rowptr_rebase(const void* in, int idx64, int64_t r0, int64_t n1, int64_t base, int64_t* out,
                          cudaStream_t s);
-// starts: scratch of validate_words(M.nnz) words (the row-start bitmap).
-int64_t validate_words(int64_t nnz);
-int launch_validate(const DevCsr& M, uint32_t* starts, uint32_t* err, cudaStream_t s);
-int launch_count(const DevCsr& A, const DevCsr& B, ClassParams cp, int64_t* P, int32_t* nnz_row,
-                  int32_t* tile_hist, int64_t* tile_sum, int64_t* tile_max, cudaStream_t s);
+// Canonical-CSR check; rp_out (may be null) receives the row pointers as int64.
+int launch_validate(const void* rp, int rp64, int64_t rows, int64_t cols, int64_t nnz, const int32_t* col,
+                    int64_t* rp_out, uint32_t* err, cudaStream_t s);
+// P_i of every row, its symbolic class, and (check) the canonical-CSR check of A; a64 (may be null)
+// receives A's row pointers as int64.
+int launch_count(const CsrArrays& A, const CsrArrays& B, int check, int64_t* a64, ClassParams cp, int64_t* P,
+                 int32_t* nnz_row, int32_t* tile_hist, int64_t* tile_sum, int64_t* tile_max, uint32_t* err,
+                 cudaStream_t s);
 int launch_class_scan(int64_t ntiles, int nclasses, int32_t* tile_hist, const int64_t* tile_sum,
                        const int64_t* tile_max, int64_t* tile_sum_off, Summary* summary,
                        cudaStream_t s);

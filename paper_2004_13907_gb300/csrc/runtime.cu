@@ -255,18 +255,24 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
              (p->abase ? m <= kSmallMaxBatchRows && p->width > 0 && p->width <= kSmallMaxCols
                        : small_path_fits(m, n));
   if (p->small) return plan_small(p, A, B, s);
+  // A and B given as the same arrays (C = A*A) have one pattern: it is converted and checked once
+  const bool same = A->row_ptr == B->row_ptr && A->col == B->col && A->rows == B->rows && A->cols == B->cols &&
+                    A->nnz == B->nnz && A->idx64_rowptr == B->idx64_rowptr;
+  int64_t* a64 = nullptr;
+  int64_t* b64 = nullptr;
   if (!A->idx64_rowptr) {
-    int64_t* t = ws_get<int64_t>(p, m + 1, &st);
+    a64 = ws_get<int64_t>(p, m + 1, &st);
     if (st) return st;
-    conv += launch_rowptr_to64(static_cast<const int32_t*>(A->row_ptr), t, m + 1, s);
-    arp = t;
+    arp = a64;
   }
   if (!B->idx64_rowptr) {
-    int64_t* t = ws_get<int64_t>(p, B->rows + 1, &st);
+    if (!same) b64 = ws_get<int64_t>(p, B->rows + 1, &st);
     if (st) return st;
-    conv += launch_rowptr_to64(static_cast<const int32_t*>(B->row_ptr), t, B->rows + 1, s);
-    brp = t;
+    brp = same ? arp : b64;
   }
+  // (the count pass copies A's row pointers and checks A; an A without rows has no count pass)
+  if (a64 && m == 0) conv += launch_rowptr_to64(static_cast<const int32_t*>(A->row_ptr), a64, 1, s);
+  if (b64 && !o.validate) conv += launch_rowptr_to64(static_cast<const int32_t*>(B->row_ptr), b64, B->rows + 1, s);
   p->A = DevCsr{m, A->cols, A->nnz, arp, A->col, A->val};
   p->B = DevCsr{B->rows, n, B->nnz, brp, B->col, B->val};
   if (p->width <= 0) p->width = n;
@@ -308,20 +314,21 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
 
   Summary h;
   if (o.validate) {
-    uint32_t* starts = ws_get<uint32_t>(p, validate_words(A->nnz > B->nnz ? A->nnz : B->nnz), &st);
-    if (st) return st;
-    // no wait here: the count kernels clamp every access, and the error word is read with the
-    // plan's summary below (an invalid input is reported before any other pass runs)
-    conv += launch_validate(p->A, starts, &p->summary->err, s);
-    conv += launch_validate(p->B, starts, &p->summary->err, s);
-    stage_end(p, SPGEMM_STAGE_VALIDATE, conv, s);
+    // no wait here: the count pass clamps every access, and the error word is read with the plan's
+    // summary below (an invalid input is reported before any other pass runs)
+    if (m == 0)
+      conv += launch_validate(A->row_ptr, A->idx64_rowptr, m, A->cols, A->nnz, A->col, nullptr, &p->summary->err, s);
+    if (!same)
+      conv += launch_validate(B->row_ptr, B->idx64_rowptr, B->rows, n, B->nnz, B->col, b64, &p->summary->err, s);
     if ((st = cuda_status(cudaGetLastError(), "launching validation")) != SPGEMM_OK) return st;
-  } else {
-    stage_end(p, SPGEMM_STAGE_VALIDATE, conv, s);
   }
+  stage_end(p, SPGEMM_STAGE_VALIDATE, conv, s);
   if (m > 0) {
     stage_begin(p, SPGEMM_STAGE_COUNT, s);
-    int nl = launch_count(p->A, p->B, p->cp, p->P, p->nnz_row, p->tile_hist, p->tile_sum, p->tile_max, s);
+    const CsrArrays ca{m, A->cols, A->nnz, A->row_ptr, A->idx64_rowptr, A->col};
+    const CsrArrays cb{B->rows, n, B->nnz, B->row_ptr, B->idx64_rowptr, B->col};
+    int nl = launch_count(ca, cb, o.validate, a64, p->cp, p->P, p->nnz_row, p->tile_hist, p->tile_sum, p->tile_max,
+                          &p->summary->err, s);
     nl += launch_class_scan(p->ntiles, kSymNumClasses, p->tile_hist, p->tile_sum, p->tile_max, nullptr,
                             p->summary, s);
     nl += launch_scatter_sym(p->A, p->cp, p->P, p->tile_hist, p->perm_s, s);
@@ -467,13 +474,12 @@ spgemm_status symbolic_run(spgemm_plan_s* p, cudaStream_t s) {
 }
 
 void plan_bytes_bounds(int64_t m, int64_t a_nnz, int64_t width, int a_rowptr32, int b_rowptr32, int64_t b_rows,
-                       int64_t b_nnz, int validate, int32_t wbits_mb, int64_t* lo, int64_t* hi) {
+                       int32_t wbits_mb, int64_t* lo, int64_t* hi) {
   const int64_t ntiles = (m + kTileRows - 1) / kTileRows;
   int64_t fixed = ws_rounded(sizeof(Summary)) + ws_rounded(16 * 4) + ws_rounded(8 * m) + 3 * ws_rounded(4 * m) +
                   ws_rounded(8 * (m + 1));
   if (a_rowptr32) fixed += ws_rounded(8 * (m + 1));
   if (b_rowptr32) fixed += ws_rounded(8 * (b_rows + 1));
-  if (validate) fixed += ws_rounded(4 * validate_words(a_nnz > b_nnz ? a_nnz : b_nnz));
   const int64_t tiles = ws_rounded(4 * ntiles * kMaxClasses) + 3 * ws_rounded(8 * ntiles);
   const int64_t nblocks = (width + kBlockCols - 1) / kBlockCols;
   const int64_t stored_words = wbits_mb > 0 ? (int64_t(wbits_mb) << 20) / 4 : 0;
