@@ -229,14 +229,19 @@ spgemm_status spgemm_plan_get_info(const spgemm_plan_t* plan, spgemm_plan_info* 
   info->products = plan->total_products;
   info->nnz_c = plan->state >= 1 ? plan->nnz_c : -1;
   info->max_row_products = plan->max_row_products;
-  for (int c = 0; c < kSymNumClasses; ++c) info->sym_class_rows[c] = plan->sym_off[c + 1] - plan->sym_off[c];
-  if (plan->state >= 1) {
-    for (int c = 0; c < kNumNumClasses; ++c) {
-      info->num_class_rows[c] = plan->num_off[c + 1] - plan->num_off[c];
-      info->num_class_products[c] = static_cast<int64_t>(plan->cls_sums[c][0]);
-      info->num_class_annz[c] = static_cast<int64_t>(plan->cls_sums[c][1]);
-      info->num_class_cnnz[c] = static_cast<int64_t>(plan->cls_sums[c][2]);
-    }
+  // the classes as the header lists them: merge rows count with the warp tables they come from
+  int q = -1;
+  for (int c = 0; c < kSymNumClasses; ++c) {
+    if (c != kSymMerge) ++q;
+    info->sym_class_rows[q] += plan->sym_off[c + 1] - plan->sym_off[c];
+  }
+  q = -1;
+  for (int c = 0; plan->state >= 1 && c < kNumNumClasses; ++c) {
+    if (c != kNumMerge1 && c != kNumMerge2) ++q;
+    info->num_class_rows[q] += plan->num_off[c + 1] - plan->num_off[c];
+    info->num_class_products[q] += static_cast<int64_t>(plan->cls_sums[c][0]);
+    info->num_class_annz[q] += static_cast<int64_t>(plan->cls_sums[c][1]);
+    info->num_class_cnnz[q] += static_cast<int64_t>(plan->cls_sums[c][2]);
   }
   info->workspace_bytes = plan->ws.total;
   info->f32c_rerun_rows = plan->f32c_rerun_rows;

@@ -19,6 +19,7 @@ enum : uint32_t {
 };
 
 constexpr int kMicroNa = 8;   // micro rows: at most this many A entries (B rows merged per thread)
+constexpr int kMergeMax = 64; // rows of as many A entries with up to this many products can be merged too
 
 // Row classes. A row's class fixes the kernel that handles it. The class order is the
 // order of the rows in the permutation, so the windowed classes come first, largest
@@ -32,6 +33,7 @@ enum SymClass : int {
   kSymWarp3,      // warp table of 2048 keys (min(P_i,n) <= 1024)
   kSymWarp2,      // warp table of 512 keys  (<= 256)
   kSymWarp1,      // warp table of 128 keys  (<= 64)
+  kSymMerge,      // of these, FP64, nnz(A_i) <= kMicroNa and P_i <= kMergeMax
   kSymTiny,       // P_i <= tiny_max and nnz(A_i) <= 32: registers only, one warp per row
   kSymMicro,      // tiny with nnz(A_i) <= kMicroNa: one thread per row merges the B rows
   kSymZero,       // P_i == 0
@@ -47,7 +49,9 @@ enum NumClass : int {
   kNumBlock1,     // block hash of 2048 slots (nnz <= 1024)
   kNumWarp3,      // warp hash of 1024 slots (nnz <= 512)
   kNumWarp2,      // warp hash of 256 slots  (nnz <= 128)
+  kNumMerge2,     // of these, FP64, nnz(A_i) <= kMicroNa and P_i <= kMergeMax
   kNumWarp1,      // warp hash of 64 slots   (nnz <= 32)
+  kNumMerge1,     // of these, the same
   kNumTiny,
   kNumMicro,      // tiny with nnz(A_i) <= kMicroNa, FP64: one thread per row merges the B rows
   kNumZero,
@@ -62,6 +66,7 @@ struct ClassParams {
   int32_t block_max;      // block tables take <= block_max; larger rows are windowed
   int32_t force_window;
   int32_t window_all;     // every row that is not tiny takes the windowed path (FP32-compensated)
+  int32_t merge;          // FP64: the merge classes are in use
   const int32_t* rwidth;  // per-row column count of C (device, NULL: every row has n columns)
 };
 
@@ -82,7 +87,7 @@ __host__ __device__ inline int sym_class(int64_t P, int32_t na, const ClassParam
   if (cp.force_window) return kSymWin0 + win_subclass(P);
   if (P <= cp.tiny_max && na <= kWarp) return na <= kMicroNa ? kSymMicro : kSymTiny;
   if (cp.window_all) return kSymWin0 + win_subclass(P);
-  if (U <= 64 && cp.warp_max >= 64) return kSymWarp1;
+  if (U <= 64 && cp.warp_max >= 64) return cp.merge && na <= kMicroNa && P <= kMergeMax ? kSymMerge : kSymWarp1;
   if (U <= 256 && cp.warp_max >= 256) return kSymWarp2;
   if (U <= cp.warp_max) return kSymWarp3;
   if (U <= cp.block_max) return kSymBlock;
@@ -95,8 +100,9 @@ __host__ __device__ inline int num_class(int64_t P, int32_t na, int32_t nnz,
   if (cp.force_window) return kNumWin0 + win_subclass(P);
   if (P <= cp.tiny_max && na <= kWarp) return (na <= kMicroNa && !cp.window_all) ? kNumMicro : kNumTiny;
   if (cp.window_all) return kNumWin0 + win_subclass(P);
-  if (nnz <= 32 && cp.warp_max >= 64) return kNumWarp1;
-  if (nnz <= 128 && cp.warp_max >= 256) return kNumWarp2;
+  const bool merge = cp.merge && na <= kMicroNa && P <= kMergeMax;
+  if (nnz <= 32 && cp.warp_max >= 64) return merge ? kNumMerge1 : kNumWarp1;
+  if (nnz <= 128 && cp.warp_max >= 256) return merge ? kNumMerge2 : kNumWarp2;
   if (nnz <= 512 && cp.warp_max >= 1024) return kNumWarp3;
   if (nnz <= 1024 && cp.block_max >= 1024) return kNumBlock1;
   if (nnz <= cp.block_max) return kNumBlock2;

@@ -123,63 +123,183 @@ __global__ void __launch_bounds__(256) k_num_tiny(DevCsr A, DevCsr B, const int3
   }
 }
 
-// Micro rows (nnz(A_i) <= kMicroNa, P_i <= tiny_max), FP64: one thread per row merges the row's
-// sorted B rows head by head. The smallest head column is the next column of C; the products of
-// every head holding it are summed in A-entry order and those heads advance. The output comes out
-// sorted, with no shared memory and no atomics.
-__global__ void __launch_bounds__(256) k_num_micro(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
-                                                   int64_t count, const int64_t* __restrict__ c_off,
-                                                   int32_t* __restrict__ ccol, double* __restrict__ cval,
-                                                   const int32_t* __restrict__ abase, uint32_t* err) {
-  constexpr int NA = kMicroNa;
+// Micro and merge rows (nnz(A_i) <= kMicroNa, P_i <= maxp <= kMergeMax), FP64: one thread per row merges
+// the columns of the row's sorted B rows head by head: the smallest head column is the next column of
+// C, and every head holding it advances. The output comes out sorted, with no hash table and no atomics;
+// the products of a column are summed in A-entry order.
+//
+// When the warp's 32 rows follow one another in C and fit `cap` entries (neighbouring rows of a stencil
+// do), the merge notes each product's place in its row and the columns are put together in shared memory
+// and leave as one run; then each thread takes the values of its B rows one row after the other, adds
+// their products at the noted places in shared memory, and the values leave as one run. Other rows
+// store from the merge.
+//
+// Bound by the L1 accesses, each lane's a B row apart. A merge that also read the values went back to
+// every B row's values after all the others', beyond what L1 holds for the warps of an SM, and stored
+// each lane's entries a row of C apart. 1024^2 five-point stencil (13.6e6 entries) 152 -> 104 us;
+// 97^3 seven-point stencil, whose 49 products a row took a 64-slot hash table and a bitonic sort, 1295
+// -> 207 us (416 with a merge of columns and values).
+constexpr int kMicroWarps = 4;
+constexpr int kMicroStaged = 8;   // mean entries of a row from which they are staged
+__host__ __device__ inline int micro_warp_bytes(int cap, int maxp) { return cap * 8 + maxp * 32; }
+
+// The first U products (of the `m` there are, possibly none) of one B row at bv, times av, added at
+// their places in the row of `len` entries at dval. The places of one B row's products differ, so all
+// are loaded before any is added.
+template <int U>
+__device__ __forceinline__ void add_head(const double* __restrict__ bv, int32_t m, double av, const uint8_t* place,
+                                         double* dval, int len) {
+  double v[U], x[U];
+  int t[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) v[u] = u < m ? bv[u] : 0.0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    t[u] = u < m ? place[u * 32] : len;
+    x[u] = t[u] < len ? dval[t[u]] : 0.0;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (t[u] < len) dval[t[u]] = x[u] + av * v[u];
+}
+
+// The rows of a warp, at most `most` <= NA entries of A in any of them (na: this lane's row's).
+template <int NA, bool Staged>
+__device__ __forceinline__ void micro_rows(const DevCsr& A, const DevCsr& B, unsigned char* mem, int cap, int maxp,
+                                           int64_t a0, int na, int most, int64_t off, int len, int32_t cb,
+                                           bool mine,
+                                           int32_t* __restrict__ ccol, double* __restrict__ cval, uint32_t* err) {
   constexpr int32_t kEnd = 0x7fffffff;
+  const int lane = threadIdx.x & 31;
+  double* sval = reinterpret_cast<double*>(mem);       // the warp's values, after
+  int32_t* scol = reinterpret_cast<int32_t*>(mem);     //   its columns
+  uint8_t* place = mem + cap * 8 + lane;               // [product * 32]: its place in the lane's row
   const double* av64 = static_cast<const double*>(A.val);
   const double* bv64 = static_cast<const double*>(B.val);
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < count; r += stride) {
-    const int32_t i = perm[r];
-    const int64_t a0 = A.rp[i];
-    const int na = static_cast<int>(A.rp[i + 1] - a0);
-    int64_t out = c_off[i];
-    const int64_t out_end = c_off[i + 1];
-    const int32_t cb = abase ? abase[i] : 0;
-    int64_t pos[NA];
-    int32_t left[NA], hc[NA];
-    double av[NA];
+  // products numbered head by head: head h holds numbers [q[h], qe[h]), product q is entry q + at[h] of B
+  int64_t at[NA];
+  int32_t q[NA], qe[NA], hc[NA];
+  int32_t products = 0;
 #pragma unroll
-    for (int h = 0; h < NA; ++h) {
-      pos[h] = 0; left[h] = 0; hc[h] = kEnd; av[h] = 0.0;
-      if (h < na) {
-        const int32_t k = A.col[a0 + h];
-        av[h] = av64[a0 + h];
-        pos[h] = B.rp[k];
-        left[h] = static_cast<int32_t>(B.rp[k + 1] - pos[h]);
-      }
+  for (int h = 0; h < NA; ++h) {
+    at[h] = 0;
+    qe[h] = 0;
+    if (h < na) {
+      const int32_t k = A.col[a0 + h];
+      at[h] = B.rp[k];
+      qe[h] = static_cast<int32_t>(B.rp[k + 1] - at[h]);
     }
+  }
 #pragma unroll
-    for (int h = 0; h < NA; ++h) if (left[h] > 0) hc[h] = B.col[pos[h]];
+  for (int h = 0; h < NA; ++h) {
+    hc[h] = qe[h] > 0 ? B.col[at[h]] : kEnd;
+    q[h] = products;
+    at[h] -= products;
+    products += qe[h];
+    qe[h] = products;
+  }
+  const int incl = warp_incl_scan(len);
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  const int64_t off0 = __shfl_sync(0xffffffffu, off, 0);
+  const bool staged =
+      Staged && total <= cap && __all_sync(0xffffffffu, products <= maxp && (!mine || off == off0 + (incl - len)));
+  int n = 0;
+  if (staged) {
+    int32_t* dcol = scol + (incl - len);
     for (;;) {
       int32_t m = hc[0];
 #pragma unroll
-      for (int h = 1; h < NA; ++h) m = hc[h] < m ? hc[h] : m;
+      for (int h = 1; h < NA; ++h) m = min(m, hc[h]);
+      if (m == kEnd) break;
+#pragma unroll
+      for (int h = 0; h < NA; ++h) {
+        if (hc[h] == m) {
+          place[q[h] * 32] = static_cast<uint8_t>(n);
+          ++q[h];
+          hc[h] = q[h] < qe[h] ? B.col[at[h] + q[h]] : kEnd;
+        }
+      }
+      if (n < len) dcol[n] = m - cb;   // a miscount raises kErrCount, never writes out of the row
+      ++n;
+    }
+    __syncwarp();
+    for (int t = lane; t < total; t += 32) ccol[off0 + t] = scol[t];
+    __syncwarp();
+    for (int t = lane; t < total; t += 32) sval[t] = 0.0;
+    __syncwarp();
+    double* dval = sval + (incl - len);
+    // the heads one after the other; the longest of the warp's B rows sets how many values are loaded
+    // together
+    int32_t p = 0;
+    int32_t k = na > 0 ? A.col[a0] : 0;
+    for (int h = 0; h < most; ++h) {
+      const bool has = h < na;
+      const double av = has ? av64[a0 + h] : 0.0;
+      const int64_t s = has ? B.rp[k] : 0;
+      const int32_t m = has ? static_cast<int32_t>(B.rp[k + 1] - s) : 0;
+      if (h + 1 < na) k = A.col[a0 + h + 1];
+      const int longest = __reduce_max_sync(0xffffffffu, m);
+      const uint8_t* pl = place + p * 32;
+      if (longest <= 1) add_head<1>(bv64 + s, m, av, pl, dval, len);
+      else if (longest <= 3) add_head<3>(bv64 + s, m, av, pl, dval, len);
+      else if (longest <= 5) add_head<5>(bv64 + s, m, av, pl, dval, len);
+      else
+        for (int32_t t = 0; t < longest; t += 8) add_head<8>(bv64 + s + t, m - t, av, pl + t * 32, dval, len);
+      p += m;
+    }
+    __syncwarp();
+    for (int t = lane; t < total; t += 32) cval[off0 + t] = sval[t];
+    __syncwarp();
+  } else {
+    double av[NA];
+#pragma unroll
+    for (int h = 0; h < NA; ++h) av[h] = h < na ? av64[a0 + h] : 0.0;
+    for (;;) {
+      int32_t m = hc[0];
+#pragma unroll
+      for (int h = 1; h < NA; ++h) m = min(m, hc[h]);
       if (m == kEnd) break;
       double sum = 0.0;
 #pragma unroll
       for (int h = 0; h < NA; ++h) {
         if (hc[h] == m) {
-          sum += av[h] * bv64[pos[h]];
-          ++pos[h];
-          --left[h];
-          hc[h] = left[h] > 0 ? B.col[pos[h]] : kEnd;
+          sum += av[h] * bv64[at[h] + q[h]];
+          ++q[h];
+          hc[h] = q[h] < qe[h] ? B.col[at[h] + q[h]] : kEnd;
         }
       }
-      if (out < out_end) {   // a miscount raises kErrCount, never writes out of the row
-        ccol[out] = m - cb;
-        cval[out] = sum;
+      if (n < len) {
+        ccol[off + n] = m - cb;
+        cval[off + n] = sum;
       }
-      ++out;
+      ++n;
     }
-    if (out != out_end) set_error(err, kErrCount);
+  }
+  if (n != len) set_error(err, kErrCount);
+}
+
+// Staged: with room for the warps' rows in shared memory; else every row is stored from the merge.
+template <bool Staged>
+__global__ void __launch_bounds__(kMicroWarps * 32, Staged ? 6 : 8) k_num_micro(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
+                                                   int64_t count, int cap, int maxp, const int64_t* __restrict__ c_off,
+                                                   int32_t* __restrict__ ccol, double* __restrict__ cval,
+                                                   const int32_t* __restrict__ abase, uint32_t* err) {
+  extern __shared__ double smem_f64[];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  unsigned char* mem = reinterpret_cast<unsigned char*>(smem_f64) + wid * micro_warp_bytes(cap, maxp);
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  for (int64_t r0 = blockIdx.x * int64_t(blockDim.x) + wid * 32; r0 < count; r0 += stride) {
+    const bool mine = r0 + lane < count;
+    const int32_t i = perm[mine ? r0 + lane : r0];
+    const int64_t a0 = A.rp[i];
+    const int na = mine ? static_cast<int>(A.rp[i + 1] - a0) : 0;
+    const int64_t off = c_off[i];
+    const int len = mine ? static_cast<int>(c_off[i + 1] - off) : 0;
+    const int32_t cb = abase ? abase[i] : 0;
+    const int most = __reduce_max_sync(0xffffffffu, na);   // heads no row of the warp has are left out
+    if (most <= 5) micro_rows<5, Staged>(A, B, mem, cap, maxp, a0, na, most, off, len, cb, mine, ccol, cval, err);
+    else if (most <= 7) micro_rows<7, Staged>(A, B, mem, cap, maxp, a0, na, most, off, len, cb, mine, ccol, cval, err);
+    else micro_rows<kMicroNa, Staged>(A, B, mem, cap, maxp, a0, na, most, off, len, cb, mine, ccol, cval, err);
   }
 }
 
@@ -735,11 +855,23 @@ int launch_num_tiny(int mode, const DevCsr& A, const DevCsr& B, const int32_t* p
   return 1;
 }
 
-int launch_num_micro(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
-                     const int64_t* c_off, int32_t* ccol, double* cval, const int32_t* abase, uint32_t* err,
-                     int num_sms, cudaStream_t s) {
+int launch_num_micro(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count, int64_t entries, int maxp,
+                     const int64_t* c_off, int32_t* ccol, double* cval, const int32_t* abase, uint32_t* err, int num_sms,
+                     cudaStream_t s) {
   if (count <= 0) return 0;
-  k_num_micro<<<grid_rows(count, 256, num_sms * 16), 256, 0, s>>>(A, B, perm, count, c_off, ccol, cval, abase, err);
+  // Room for 32 rows a sixteenth longer than the mean: regular rows fit, and an SM holds many warps.
+  // Rows of fewer entries are stored from the merge, whose lanes are then close together (A*P of the
+  // Galerkin set-up, 3 entries a row: 41 us against 59).
+  const int64_t mean = (entries + count - 1) / count;
+  const int cap = static_cast<int>((32 * mean + 2 * mean + 31) & ~int64_t(31));
+  const size_t sm = size_t(kMicroWarps) * micro_warp_bytes(cap, maxp);   // at most 4 x 19,456 bytes
+  auto go = [&](auto kernel, size_t smem) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    kernel<<<grid_rows(count, kMicroWarps * 32, num_sms * 32), kMicroWarps * 32, smem, s>>>(A, B, perm, count, cap, maxp,
+                                                                                           c_off, ccol, cval, abase, err);
+  };
+  if (mean >= kMicroStaged) go(k_num_micro<true>, sm);
+  else go(k_num_micro<false>, 0);
   return 1;
 }
 

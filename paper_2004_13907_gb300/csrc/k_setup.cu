@@ -161,6 +161,37 @@ __device__ __forceinline__ int32_t aggregated_slot(int32_t* counters, int cls, b
   return base + rank;
 }
 
+// Places of 256 consecutive rows (one per thread) within their classes, in row order, from base[class],
+// which moves past them: neighbouring rows of a class stay neighbours in the permutation (the merge
+// kernel writes a warp's rows as one run). cnt: a counter per warp and class. Contains __syncthreads.
+__device__ __forceinline__ int32_t ordered_slot(int32_t* base, int32_t (*cnt)[kMaxClasses], int cls, bool valid) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane < kMaxClasses) cnt[wid][lane] = 0;
+  __syncwarp();
+  unsigned peers = 0;
+  for (unsigned todo = __ballot_sync(0xffffffffu, valid); todo;) {
+    const int lc = __shfl_sync(0xffffffffu, cls, __ffs(todo) - 1);
+    const unsigned same = __ballot_sync(0xffffffffu, valid && cls == lc);
+    if (valid && cls == lc) peers = same;
+    if (lane == 0) cnt[wid][lc] = __popc(same);
+    todo &= ~same;
+  }
+  __syncthreads();
+  int32_t at = 0;
+  if (valid) {
+    at = base[cls] + __popc(peers & ((1u << lane) - 1u));
+    for (int w = 0; w < wid; ++w) at += cnt[w][cls];
+  }
+  __syncthreads();
+  if (threadIdx.x < kMaxClasses) {
+    int32_t all = 0;
+    for (int w = 0; w < 8; ++w) all += cnt[w][threadIdx.x];
+    base[threadIdx.x] += all;
+  }
+  __syncthreads();
+  return at;
+}
+
 // Rows with more entries than this are counted by the whole block of k_count.
 constexpr int64_t kCountBlockNa = 2048;
 
@@ -383,6 +414,7 @@ __global__ void __launch_bounds__(544) k_class_scan(int64_t ntiles, int nclasses
 __global__ void __launch_bounds__(256) k_scatter_sym(DevCsr A, ClassParams cp, const int64_t* P,
                                                      const int32_t* tile_hist, int32_t* perm) {
   __shared__ int32_t base[kMaxClasses];
+  __shared__ int32_t s_cnt[8][kMaxClasses];
   const int64_t t = blockIdx.x;
   if (threadIdx.x < kMaxClasses) base[threadIdx.x] = tile_hist[threadIdx.x * int64_t(gridDim.x) + t];
   __syncthreads();
@@ -395,7 +427,7 @@ __global__ void __launch_bounds__(256) k_scatter_sym(DevCsr A, ClassParams cp, c
       clamped_row(A, row, a0, na);   // the same row length k_count classified (before validation's verdict)
       cls = sym_class(P[row], na > 0x7fffffff ? 0x7fffffff : static_cast<int32_t>(na), row_params(cp, row));
     }
-    const int32_t pos = aggregated_slot(base, cls, valid);
+    const int32_t pos = ordered_slot(base, s_cnt, cls, valid);
     if (valid) perm[pos] = static_cast<int32_t>(row);
   }
 }
@@ -461,6 +493,7 @@ __global__ void __launch_bounds__(256) k_scatter_num(DevCsr A, ClassParams cp, c
                                                      const int64_t* tile_sum_off, int32_t* perm,
                                                      int64_t* c_off) {
   __shared__ int32_t base[kMaxClasses];
+  __shared__ int32_t s_cnt[8][kMaxClasses];
   __shared__ int64_t scratch[33];
   const int64_t t = blockIdx.x;
   if (threadIdx.x < kMaxClasses) base[threadIdx.x] = tile_hist[threadIdx.x * int64_t(gridDim.x) + t];
@@ -484,7 +517,7 @@ __global__ void __launch_bounds__(256) k_scatter_num(DevCsr A, ClassParams cp, c
       if (row == A.rows - 1) c_off[A.rows] = carry + ex + z;
     }
     carry += tot;
-    const int32_t pos = aggregated_slot(base, cls, valid);
+    const int32_t pos = ordered_slot(base, s_cnt, cls, valid);
     if (valid) perm[pos] = static_cast<int32_t>(row);
   }
 }

@@ -56,48 +56,59 @@ __global__ void __launch_bounds__(256) k_sym_tiny(DevCsr A, DevCsr B, const int3
   }
 }
 
-// Micro rows (nnz(A_i) <= kMicroNa, P_i <= tiny_max): one thread per row merges the row's sorted
-// B rows head by head (the smallest head column is the next column of C; every head holding it
-// advances) and counts the distinct columns.
-__global__ void __launch_bounds__(256) k_sym_micro(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
-                                                   int64_t count, int32_t* __restrict__ nnz_row) {
-  constexpr int NA = kMicroNa;
+// Micro and merge rows (nnz(A_i) <= kMicroNa): one thread per row merges the row's sorted B rows head
+// by head (the smallest head column is the next column of C; every head holding it advances) and
+// counts the distinct columns. NA: the most A entries of a row of the warp.
+template <int NA>
+__device__ __forceinline__ int32_t merge_count(const DevCsr& A, const DevCsr& B, int64_t a0, int na) {
   constexpr int32_t kEnd = 0x7fffffff;   // column of an exhausted head (every column is smaller)
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < count; r += stride) {
-    const int32_t i = perm[r];
-    const int64_t a0 = A.rp[i];
-    const int na = static_cast<int>(A.rp[i + 1] - a0);
-    int64_t pos[NA];
-    int32_t left[NA], hc[NA];
+  int64_t pos[NA];
+  int32_t left[NA], hc[NA];
+#pragma unroll
+  for (int h = 0; h < NA; ++h) {
+    pos[h] = 0; left[h] = 0; hc[h] = kEnd;
+    if (h < na) {
+      const int32_t k = A.col[a0 + h];
+      pos[h] = B.rp[k];
+      left[h] = static_cast<int32_t>(B.rp[k + 1] - pos[h]);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < NA; ++h) if (left[h] > 0) hc[h] = B.col[pos[h]];
+  int32_t n = 0;
+  for (;;) {
+    int32_t m = hc[0];
+#pragma unroll
+    for (int h = 1; h < NA; ++h) m = min(m, hc[h]);
+    if (m == kEnd) break;
+    ++n;
 #pragma unroll
     for (int h = 0; h < NA; ++h) {
-      pos[h] = 0; left[h] = 0; hc[h] = kEnd;
-      if (h < na) {
-        const int32_t k = A.col[a0 + h];
-        pos[h] = B.rp[k];
-        left[h] = static_cast<int32_t>(B.rp[k + 1] - pos[h]);
+      if (hc[h] == m) {
+        ++pos[h];
+        --left[h];
+        hc[h] = left[h] > 0 ? B.col[pos[h]] : kEnd;
       }
     }
-#pragma unroll
-    for (int h = 0; h < NA; ++h) if (left[h] > 0) hc[h] = B.col[pos[h]];
-    int32_t n = 0;
-    for (;;) {
-      int32_t m = hc[0];
-#pragma unroll
-      for (int h = 1; h < NA; ++h) m = hc[h] < m ? hc[h] : m;
-      if (m == kEnd) break;
-      ++n;
-#pragma unroll
-      for (int h = 0; h < NA; ++h) {
-        if (hc[h] == m) {
-          ++pos[h];
-          --left[h];
-          hc[h] = left[h] > 0 ? B.col[pos[h]] : kEnd;
-        }
-      }
-    }
-    nnz_row[i] = n;
+  }
+  return n;
+}
+
+__global__ void __launch_bounds__(256) k_sym_micro(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
+                                                   int64_t count, int32_t* __restrict__ nnz_row) {
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  for (int64_t r0 = blockIdx.x * int64_t(blockDim.x) + (threadIdx.x & ~31); r0 < count; r0 += stride) {
+    const int64_t r = r0 + (threadIdx.x & 31);
+    const bool mine = r < count;
+    const int32_t i = perm[mine ? r : r0];
+    const int64_t a0 = A.rp[i];
+    const int na = mine ? static_cast<int>(A.rp[i + 1] - a0) : 0;
+    const int most = __reduce_max_sync(0xffffffffu, na);
+    int32_t n;
+    if (most <= 5) n = merge_count<5>(A, B, a0, na);
+    else if (most <= 7) n = merge_count<7>(A, B, a0, na);
+    else n = merge_count<kMicroNa>(A, B, a0, na);
+    if (mine) nnz_row[i] = n;
   }
 }
 

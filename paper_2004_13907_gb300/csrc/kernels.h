@@ -137,7 +137,8 @@ int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int
 int launch_num_tiny(int mode, const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
                     const int64_t* c_off, int32_t* ccol, void* cval, int32_t* row_flag, const int32_t* abase,
                     uint32_t* err, int num_sms, cudaStream_t s);
-int launch_num_micro(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
+// entries: entries of C of all these rows; maxp: partial products of a row at most.
+int launch_num_micro(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count, int64_t entries, int maxp,
                      const int64_t* c_off, int32_t* ccol, double* cval, const int32_t* abase, uint32_t* err,
                      int num_sms, cudaStream_t s);
 // Warp and block hash kernels, kModeF64 or kModeF32C (row_flag lists kModeF32C rows for the FP64

@@ -284,6 +284,7 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
   // deterministic FP64 (fp64_accumulate 2): every non-empty row takes the exact windowed path
   p->cp.force_window = (o.force_window || (p->prec == SPGEMM_F64 && o.fp64_accumulate == 2)) ? 1 : 0;
   p->cp.window_all = p->prec == SPGEMM_F32_COMPENSATED ? 1 : 0;
+  p->cp.merge = p->prec == SPGEMM_F64 ? 1 : 0;
   if (o.window_hash_fill < 1 || o.window_hash_fill > 4096) p->opts.window_hash_fill = 4096;
 
   p->ntiles = (m + kTileRows - 1) / kTileRows;
@@ -439,7 +440,11 @@ spgemm_status symbolic_run(spgemm_plan_s* p, cudaStream_t s) {
     stage_begin(p, SPGEMM_STAGE_SYM_WARP, s);
     nl = launch_sym_warp(11, p->A, p->B, seg(kSymWarp3), cnt(kSymWarp3), p->nnz_row, err, p->num_sms, s);
     nl += launch_sym_warp(9, p->A, p->B, seg(kSymWarp2), cnt(kSymWarp2), p->nnz_row, err, p->num_sms, s);
-    nl += launch_sym_warp(7, p->A, p->B, seg(kSymWarp1), cnt(kSymWarp1), p->nnz_row, err, p->num_sms, s);
+    // few merge rows stay with the warp table their class continues (kMicroMinRows)
+    const bool merge = cnt(kSymMerge) >= kMicroMinRows;
+    nl += launch_sym_warp(7, p->A, p->B, seg(kSymWarp1), cnt(kSymWarp1) + (merge ? 0 : cnt(kSymMerge)), p->nnz_row, err,
+                          p->num_sms, s);
+    if (merge) nl += launch_sym_micro(p->A, p->B, seg(kSymMerge), cnt(kSymMerge), p->nnz_row, p->num_sms, s);
     stage_end(p, SPGEMM_STAGE_SYM_WARP, nl, s);
     stage_begin(p, SPGEMM_STAGE_SYM_TINY, s);
     if (cnt(kSymMicro) < kMicroMinRows) {
@@ -689,6 +694,10 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
     nl = p->sub ? 0 : launch_expand_cols(seg(kNumWin0), nwin, p->win_slot, p->woff, p->wbits, p->blockcnt, p->nblocks, p->c_off,
                             p->awidth, p->width, C->col, p->num_sms, err, s);
     stage_end(p, SPGEMM_STAGE_NUM_EXPAND, nl, s);
+    auto micro = [&](int c) {
+      return launch_num_micro(p->A, p->B, seg(c), cnt(c), static_cast<int64_t>(p->cls_sums[c][2]),
+                              c == kNumMicro ? kWarp : kMergeMax, p->c_off, C->col, static_cast<double*>(C->val), p->abase, err, p->num_sms, s);
+    };
     {
       int32_t* flag = f32c ? p->rerun_flag : nullptr;
       const int32_t* neg = f32c ? p->counters + 8 : nullptr;
@@ -701,19 +710,20 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
       stage_begin(p, SPGEMM_STAGE_NUM_WARP, s);
       nl = launch_num_warp(10, mode, p->A, p->B, seg(kNumWarp3), cnt(kNumWarp3), p->c_off, C->col, C->val, p->abase,
                            flag, neg, err, p->num_sms, s);
-      nl += launch_num_warp(8, mode, p->A, p->B, seg(kNumWarp2), cnt(kNumWarp2), p->c_off, C->col, C->val, p->abase,
-                            flag, neg, err, p->num_sms, s);
-      nl += launch_num_warp(6, mode, p->A, p->B, seg(kNumWarp1), cnt(kNumWarp1), p->c_off, C->col, C->val, p->abase,
-                            flag, neg, err, p->num_sms, s);
+      const bool merge2 = cnt(kNumMerge2) >= kMicroMinRows, merge1 = cnt(kNumMerge1) >= kMicroMinRows;
+      nl += launch_num_warp(8, mode, p->A, p->B, seg(kNumWarp2), cnt(kNumWarp2) + (merge2 ? 0 : cnt(kNumMerge2)), p->c_off,
+                            C->col, C->val, p->abase, flag, neg, err, p->num_sms, s);
+      nl += launch_num_warp(6, mode, p->A, p->B, seg(kNumWarp1), cnt(kNumWarp1) + (merge1 ? 0 : cnt(kNumMerge1)), p->c_off,
+                            C->col, C->val, p->abase, flag, neg, err, p->num_sms, s);
+      if (merge2) nl += micro(kNumMerge2);
+      if (merge1) nl += micro(kNumMerge1);
       stage_end(p, SPGEMM_STAGE_NUM_WARP, nl, s);
     }
     stage_begin(p, SPGEMM_STAGE_NUM_TINY, s);
     const bool micro_as_tiny = f32c || cnt(kNumMicro) < kMicroMinRows;   // (F32 plans have no micro rows)
     nl = launch_num_tiny(mode, p->A, p->B, seg(kNumTiny), cnt(kNumTiny) + (micro_as_tiny ? cnt(kNumMicro) : 0),
                          p->c_off, C->col, C->val, p->rerun_flag, p->abase, err, p->num_sms, s);
-    if (!micro_as_tiny)
-      nl += launch_num_micro(p->A, p->B, seg(kNumMicro), cnt(kNumMicro), p->c_off, C->col,
-                             static_cast<double*>(C->val), p->abase, err, p->num_sms, s);
+    if (!micro_as_tiny) nl += micro(kNumMicro);
     stage_end(p, SPGEMM_STAGE_NUM_TINY, nl, s);
     if (f32c && !p->opts.f32c_rerun_none) {
       // rows with an entry over the compensated bound are recomputed in FP64 and rounded once

@@ -127,7 +127,8 @@ spgemm_status read_small(void* dst, const void* src, size_t bytes, cudaStream_t 
 void release_small_host(spgemm_plan_s* p);
 // Below this many micro rows (at most 8 A entries and 32 partial products) the rows take the
 // warp-per-row tiny kernels instead of the thread-per-row merge, whose dependent loads make it
-// pay only when many rows run at once.
+// pay only when many rows run at once; the same holds for the merge rows (up to 64 partial products)
+// and their warp tables.
 constexpr int64_t kMicroMinRows = 32768;
 // Bytes of FP64 scratch the FP32 rerun of windowed rows works in (rows of the plan's width).
 constexpr int64_t kRerunScratchBytes = int64_t(256) << 20;
