@@ -341,7 +341,12 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   bool bad = false;
   int64_t prod = 0;
   int max_cnt = 0;
-  for (int64_t gs = r0 + wid * G; gs < r1; gs += int64_t(kSymWarps) * G) {
+  // A row of C over kSmallCap entries sends the whole product to the general path: the warp that finds
+  // one says so at once, and the others, which look once per group (a load that the group's work hides),
+  // stop there. Counting on to the end took 1.8 ms of a 30,000^2 product whose every row is too long.
+  bool stop = false;
+  for (int64_t gs = r0 + wid * G; gs < r1 && !stop; gs += int64_t(kSymWarps) * G) {
+    const uint32_t flags = *reinterpret_cast<const volatile uint32_t*>(&sum->small_flags);
     const int ng = r1 - gs < G ? static_cast<int>(r1 - gs) : G;
     const RowGroup gr = group_rows(A, gs, ng, chk, bad);
     // lane g < ng: the first column of row gs + g's column space (a stacked batch's job)
@@ -384,9 +389,14 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
         max_cnt = cnt > max_cnt ? cnt : max_cnt;
       }
     }
+    if (max_cnt > kSmallCap) {
+      if (lane == 0) atomicOr(&sum->small_flags, kSmallTooLong);
+      stop = true;
+    }
+    stop |= (flags & kSmallTooLong) != 0u;
     __syncwarp();
   }
-  if (chk) {
+  if (chk && !stop) {
     // B: row pointers, columns in range and strictly increasing, 32 rows per warp at a time
     const int64_t gw = blockIdx.x * int64_t(kSymWarps) + wid;
     const int64_t nw = int64_t(gridDim.x) * kSymWarps;
@@ -412,7 +422,6 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
     if (prod) atomicAdd(&sum->small_products, static_cast<unsigned long long>(prod));
     if (max_cnt > 0)
       atomicMax(reinterpret_cast<unsigned long long*>(&sum->max_row), static_cast<unsigned long long>(max_cnt));
-    if (max_cnt > kSmallCap) atomicOr(&sum->small_flags, kSmallTooLong);
   }
   // offsets within this block's run of rows, and the run's total
   __syncthreads();
