@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "batch.h"
@@ -23,7 +24,9 @@ namespace spg {
 
 namespace {
 
-constexpr int64_t kTile = 1 << 15;
+// Rows or entries of one block of the stacking kernels. A block's 16 per thread are loaded together; with
+// 32,768 a batch of small jobs filled a few blocks only (20 jobs, 1.7e5 entries: 118 us a side, now 12).
+constexpr int64_t kTile = 1 << 12;
 
 // One stacked matrix (A or B side) of one job.
 struct Part {
@@ -49,31 +52,50 @@ struct Tile {
 __global__ void __launch_bounds__(256) k_stack(const Part* __restrict__ parts, const Tile* __restrict__ tiles,
                                                int64_t* __restrict__ rp_out, int32_t* __restrict__ col_out,
                                                unsigned char* __restrict__ val_out, int32_t* __restrict__ base_out,
-                                               int32_t* __restrict__ width_out, int val_bytes, uint32_t* err) {
+                                               int32_t* __restrict__ width_out, int val_bytes, int64_t rows,
+                                               int64_t nnz, uint32_t* err) {
+  if (rp_out && blockIdx.x == 0 && threadIdx.x == 0) rp_out[rows] = nnz;
   const Tile t = tiles[blockIdx.x];
   const Part pt = parts[t.part];
+  constexpr int kPer = static_cast<int>(kTile / 256);
   if (t.kind == 0) {
     const int64_t end = t.start + kTile < pt.rows ? t.start + kTile : pt.rows;
-    for (int64_t r = t.start + threadIdx.x; r < end; r += blockDim.x) {
+#pragma unroll 4
+    for (int64_t r = t.start + threadIdx.x; r < end; r += 256) {
       const int64_t v = pt.idx64 ? static_cast<const int64_t*>(pt.rp)[r] : static_cast<const int32_t*>(pt.rp)[r];
       rp_out[pt.row0 + r] = v + pt.nnz0;
       base_out[pt.row0 + r] = pt.base;
       if (width_out) width_out[pt.row0 + r] = pt.width;
     }
-  } else {
-    const int64_t end = t.start + kTile < pt.nnz ? t.start + kTile : pt.nnz;
-    for (int64_t e = t.start + threadIdx.x; e < end; e += blockDim.x) {
-      if (t.kind == 1) {
-        const int32_t c = pt.col[e];
-        if (c < 0 || c >= pt.col_limit) set_error(err, kErrInvalidCsr);
-        col_out[pt.nnz0 + e] = static_cast<int32_t>(c + pt.col_shift);
-      }
-      if (val_bytes == 8)
-        reinterpret_cast<double*>(val_out)[pt.nnz0 + e] = static_cast<const double*>(pt.val)[e];
-      else
-        reinterpret_cast<float*>(val_out)[pt.nnz0 + e] = static_cast<const float*>(pt.val)[e];
-    }
+    return;
   }
+  const int64_t end = t.start + kTile < pt.nnz ? t.start + kTile : pt.nnz;
+  const int64_t first = t.start + threadIdx.x;
+  if (t.kind == 1) {
+    int32_t c[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) c[u] = first + u * 256 < end ? pt.col[first + u * 256] : 0;
+    bool bad = false;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int64_t e = first + u * 256;
+      if (e >= end) continue;
+      bad |= c[u] < 0 || c[u] >= pt.col_limit;
+      col_out[pt.nnz0 + e] = static_cast<int32_t>(c[u] + pt.col_shift);
+    }
+    if (bad) set_error(err, kErrInvalidCsr);
+  }
+  auto values = [&](auto* out, const auto* in) {
+    std::remove_cv_t<std::remove_reference_t<decltype(*out)>> v[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+      if (first + u * 256 < end) v[u] = in[first + u * 256];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+      if (first + u * 256 < end) out[pt.nnz0 + first + u * 256] = v[u];
+  };
+  if (val_bytes == 8) values(reinterpret_cast<double*>(val_out), static_cast<const double*>(pt.val));
+  else values(reinterpret_cast<float*>(val_out), static_cast<const float*>(pt.val));
 }
 
 // Per-job row pointers starting at 0: out[row0_j + j + r] = c_off[row0_j + r] - c_off[row0_j].
@@ -86,6 +108,13 @@ __global__ void __launch_bounds__(256) k_job_rowptr(const Part* __restrict__ par
   const int64_t first = c_off[pt.row0];
   for (int64_t r = t.start + threadIdx.x; r < end; r += blockDim.x)
     out[pt.row0 + job + r] = c_off[pt.row0 + r] - first;
+}
+
+// Entry offset of each job: out[j] = c_off[first row of job j], out[n] = the total (row `rows`).
+__global__ void __launch_bounds__(256) k_job_offsets(const Part* __restrict__ parts, int64_t n, int64_t rows,
+                                                     const int64_t* __restrict__ c_off, int64_t* __restrict__ out) {
+  const int64_t j = blockIdx.x * int64_t(256) + threadIdx.x;
+  if (j <= n) out[j] = c_off[j < n ? parts[j].row0 : rows];
 }
 
 void add_tiles(std::vector<Tile>& tiles, int part, int kind, int64_t count) {
@@ -204,10 +233,30 @@ spgemm_status batch_prepare(int64_t n_jobs, const spgemm_csr_in* A, const spgemm
   }
   const int vb = prec == SPGEMM_F64 ? 8 : 4;
   auto get = [&](size_t bytes) { return b->ws.get(bytes); };
-  b->d_parts = static_cast<Part*>(get(sizeof(Part) * b->parts.size()));
-  b->d_stack_tiles = static_cast<Tile*>(get(sizeof(Tile) * (b->stack_tiles.size() + 1)));
-  b->d_value_tiles = static_cast<Tile*>(get(sizeof(Tile) * (b->value_tiles.size() + 1)));
-  b->d_rowptr_tiles = static_cast<Tile*>(get(sizeof(Tile) * (b->rowptr_tiles.size() + 1)));
+  // the job tables in one block: parts, the three tile lists, the last row pointers of A and B, the error
+  // word (zero), and room for the jobs' entry offsets; copied to the device at once
+  const size_t parts_b = sizeof(Part) * b->parts.size();
+  const size_t stack_b = sizeof(Tile) * b->stack_tiles.size(), value_b = sizeof(Tile) * b->value_tiles.size();
+  const size_t rowptr_b = sizeof(Tile) * b->rowptr_tiles.size();
+  std::vector<unsigned char> tables(parts_b + stack_b + value_b + rowptr_b + 8);
+  {
+    unsigned char* t = tables.data();
+    auto put = [&](const void* from, size_t bytes) {
+      if (bytes) std::memcpy(t, from, bytes);
+      t += bytes;
+    };
+    put(b->parts.data(), parts_b);
+    put(b->stack_tiles.data(), stack_b);
+    put(b->value_tiles.data(), value_b);
+    put(b->rowptr_tiles.data(), rowptr_b);
+  }
+  unsigned char* const d_tables = static_cast<unsigned char*>(get(tables.size() + 8 * (n_jobs + 1)));
+  b->d_parts = reinterpret_cast<Part*>(d_tables);
+  b->d_stack_tiles = reinterpret_cast<Tile*>(d_tables + parts_b);
+  b->d_value_tiles = reinterpret_cast<Tile*>(d_tables + parts_b + stack_b);
+  b->d_rowptr_tiles = reinterpret_cast<Tile*>(d_tables + parts_b + stack_b + value_b);
+  b->err = reinterpret_cast<uint32_t*>(d_tables + parts_b + stack_b + value_b + rowptr_b);
+  int64_t* const d_offsets = reinterpret_cast<int64_t*>(d_tables + tables.size());
   b->a_rp = static_cast<int64_t*>(get(sizeof(int64_t) * (b->rows + 1)));
   b->a_col = static_cast<int32_t*>(get(sizeof(int32_t) * b->a_nnz));
   b->a_val = get(static_cast<size_t>(vb) * b->a_nnz);
@@ -217,26 +266,12 @@ spgemm_status batch_prepare(int64_t n_jobs, const spgemm_csr_in* A, const spgemm
   b->b_col = static_cast<int32_t*>(get(sizeof(int32_t) * b->b_nnz));
   b->b_val = get(static_cast<size_t>(vb) * b->b_nnz);
   b->bbase = static_cast<int32_t*>(get(sizeof(int32_t) * b->inner));
-  b->err = static_cast<uint32_t*>(get(sizeof(uint32_t)));
-  if (!b->d_parts || !b->d_stack_tiles || !b->d_value_tiles || !b->d_rowptr_tiles || !b->a_rp || !b->a_col ||
-      !b->a_val || !b->abase || !b->awidth || !b->b_rp || !b->b_col || !b->b_val || !b->bbase || !b->err) {
+  if (!d_tables || !b->a_rp || !b->a_col || !b->a_val || !b->abase || !b->awidth || !b->b_rp || !b->b_col || !b->b_val ||
+      !b->bbase) {
     set_error_msg(SPGEMM_ERR_OOM, "device allocation of the stacked batch failed");
     return fail(SPGEMM_ERR_OOM);
   }
-  cudaError_t e = cudaMemcpyAsync(b->d_parts, b->parts.data(), sizeof(Part) * b->parts.size(),
-                                  cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && !b->stack_tiles.empty())
-    e = cudaMemcpyAsync(b->d_stack_tiles, b->stack_tiles.data(), sizeof(Tile) * b->stack_tiles.size(),
-                        cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && !b->value_tiles.empty())
-    e = cudaMemcpyAsync(b->d_value_tiles, b->value_tiles.data(), sizeof(Tile) * b->value_tiles.size(),
-                        cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess && !b->rowptr_tiles.empty())
-    e = cudaMemcpyAsync(b->d_rowptr_tiles, b->rowptr_tiles.data(), sizeof(Tile) * b->rowptr_tiles.size(),
-                        cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->err, 0, sizeof(uint32_t), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b->a_rp + b->rows, &b->a_nnz, sizeof(int64_t), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b->b_rp + b->inner, &b->b_nnz, sizeof(int64_t), cudaMemcpyHostToDevice, s);
+  cudaError_t e = cudaMemcpyAsync(d_tables, tables.data(), tables.size(), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) { cuda_status(e, "staging the batch tables"); return fail(SPGEMM_ERR_CUDA); }
   // stack A (columns shifted to the job's B rows) and B (columns shifted to the job's columns)
   {
@@ -244,12 +279,16 @@ spgemm_status batch_prepare(int64_t n_jobs, const spgemm_csr_in* A, const spgemm
     if (na > 0)
       k_stack<<<static_cast<unsigned>(na), 256, 0, s>>>(b->d_parts, b->d_stack_tiles, b->a_rp, b->a_col,
                                                         static_cast<unsigned char*>(b->a_val), b->abase, b->awidth, vb,
-                                                        b->err);
+                                                        b->rows, b->a_nnz, b->err);
     if (nb > 0)
       k_stack<<<static_cast<unsigned>(nb), 256, 0, s>>>(b->d_parts, b->d_stack_tiles + na, b->b_rp, b->b_col,
                                                         static_cast<unsigned char*>(b->b_val), b->bbase, nullptr, vb,
-                                                        b->err);
+                                                        b->inner, b->b_nnz, b->err);
     b->launches += (na > 0) + (nb > 0);
+    // no tile: no rows and no entries, one row pointer of zero
+    if (na == 0) e = cudaMemsetAsync(b->a_rp, 0, sizeof(int64_t), s);
+    if (nb == 0 && e == cudaSuccess) e = cudaMemsetAsync(b->b_rp, 0, sizeof(int64_t), s);
+    if (e != cudaSuccess) { cuda_status(e, "staging the batch"); return fail(SPGEMM_ERR_CUDA); }
   }
   uint32_t herr = 0;
   if ((st = read_small(&herr, b->err, sizeof(herr), s, &b->launches, "stacking the batch")) != SPGEMM_OK)
@@ -276,15 +315,13 @@ spgemm_status batch_prepare(int64_t n_jobs, const spgemm_csr_in* A, const spgemm
   if ((st = plan_run(p, &SA, &SB, s)) != SPGEMM_OK) return fail(st);
   if ((st = symbolic_run(p, s)) != SPGEMM_OK) return fail(st);
   // per-job entry offsets from the row offsets of C
-  std::vector<int64_t> row0(static_cast<size_t>(n_jobs) + 1);
-  for (int64_t j = 0; j < n_jobs; ++j) row0[j] = b->parts[j].row0;
-  row0[n_jobs] = b->rows;
   b->job_nnz0.resize(static_cast<size_t>(n_jobs) + 1);
-  std::vector<int64_t> h_off(static_cast<size_t>(b->rows) + 1);
-  e = cudaMemcpyAsync(h_off.data(), p->c_off, sizeof(int64_t) * (b->rows + 1), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) { cuda_status(e, "reading the batch row offsets"); return fail(SPGEMM_ERR_CUDA); }
-  for (int64_t j = 0; j <= n_jobs; ++j) b->job_nnz0[j] = h_off[row0[j]];
+  k_job_offsets<<<static_cast<unsigned>(n_jobs / 256 + 1), 256, 0, s>>>(b->d_parts, n_jobs, b->rows, p->c_off, d_offsets);
+  ++b->launches;
+  const size_t off_bytes = sizeof(int64_t) * (static_cast<size_t>(n_jobs) + 1);
+  if ((st = cuda_status(cudaGetLastError(), "launching the job offsets")) != SPGEMM_OK) return fail(st);
+  if ((st = read_small(b->job_nnz0.data(), d_offsets, off_bytes, s, &b->launches, "reading the job offsets")) != SPGEMM_OK)
+    return fail(st);
   *out = b;
   return SPGEMM_OK;
 }
@@ -304,13 +341,12 @@ void batch_prepare_bounds(int64_t n_jobs, const spgemm_csr_in* A, const spgemm_c
     value_tiles += t(A[j].nnz) + t(B[j].nnz);
     rp_tiles += t(A[j].rows + 1);
   }
-  const int64_t stacked = ws_rounded(int64_t(sizeof(Part)) * 2 * n_jobs) +
-                          ws_rounded(int64_t(sizeof(Tile)) * (stack_tiles + 1)) +
-                          ws_rounded(int64_t(sizeof(Tile)) * (value_tiles + 1)) +
-                          ws_rounded(int64_t(sizeof(Tile)) * (rp_tiles + 1)) + ws_rounded(8 * (rows + 1)) +
+  const int64_t stacked = ws_rounded(int64_t(sizeof(Part)) * 2 * n_jobs +
+                                     int64_t(sizeof(Tile)) * (stack_tiles + value_tiles + rp_tiles) + 8 + 8 * (n_jobs + 1)) +
+                          ws_rounded(8 * (rows + 1)) +
                           ws_rounded(4 * a_nnz) + ws_rounded(vb * a_nnz) + 2 * ws_rounded(4 * rows) +
                           ws_rounded(8 * (inner + 1)) + ws_rounded(4 * b_nnz) + ws_rounded(vb * b_nnz) +
-                          ws_rounded(4 * inner) + ws_rounded(4);
+                          ws_rounded(4 * inner);
   int64_t plo = 0, phi = 0;
   plan_bytes_bounds(rows, a_nnz, width, 0, 0, inner, opts->window_cols_max_mb, &plo, &phi);
   *lo = stacked + plo;
@@ -452,13 +488,13 @@ extern "C" spgemm_status spgemm_batch_replay(spgemm_batch_t* b, void* stream) {
     const int vb = 8;
     const int64_t na = b->value_a, nb = static_cast<int64_t>(b->value_tiles.size()) - b->value_a;
     if (na > 0)
-      k_stack<<<static_cast<unsigned>(na), 256, 0, cs>>>(b->d_parts, b->d_value_tiles, b->a_rp, b->a_col,
+      k_stack<<<static_cast<unsigned>(na), 256, 0, cs>>>(b->d_parts, b->d_value_tiles, nullptr, b->a_col,
                                                          static_cast<unsigned char*>(b->a_val), b->abase, nullptr, vb,
-                                                         b->err);
+                                                         b->rows, b->a_nnz, b->err);
     if (nb > 0)
-      k_stack<<<static_cast<unsigned>(nb), 256, 0, cs>>>(b->d_parts, b->d_value_tiles + na, b->b_rp, b->b_col,
+      k_stack<<<static_cast<unsigned>(nb), 256, 0, cs>>>(b->d_parts, b->d_value_tiles + na, nullptr, b->b_col,
                                                          static_cast<unsigned char*>(b->b_val), b->bbase, nullptr, vb,
-                                                         b->err);
+                                                         b->inner, b->b_nnz, b->err);
     spgemm_csr_out C{b->rows, b->cols, p->nnz_c, 1, 0, p->c_off, b->c_col, b->c_val};
     spgemm_status st = numeric_run(p, &C, cs);
     cudaGraph_t g = nullptr;
