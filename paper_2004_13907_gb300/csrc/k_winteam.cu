@@ -21,6 +21,13 @@
 // of 32 products of one segment need no search per product. Both kernels -> this one: 30,000^2
 // uniform (d = 5e-3, 6.7e8 products) 7.35 -> 5.06 ms, R-MAT 2^17 (1.09e9) 9.92 -> 6.39 ms, R-MAT 2^19
 // (7.85e9) 77.6 -> 58.5 ms.
+//
+// FP32-compensated plans take the same kernel with FP32 sums and compensations in the eight bytes of a
+// slot (two FP32 atomics a product, separate arrays so that both spread over all banks): R-MAT 2^17
+// 7.93 -> 6.12 ms. A slot that also needs the sum of |p| and the term count takes sixteen bytes and its
+// windows half the entries; with mixed signs (R-MAT 2^17 of 8 edges a vertex) 4.51 -> 3.50 ms.
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -45,7 +52,8 @@ constexpr int kRankStep = kWinSpan / 4 / kTeam;   // runs of four sub-blocks per
 constexpr int kGroups = 2;         // groups of 32 products per step; a warp has two steps under way
 constexpr int kSlots = 3;          // window records in shared memory: this one, the next, the one after
 constexpr unsigned kFull = 0xffffffffu;
-static_assert(kWinCap >= kSubCols, "a window holds any single sub-block");
+constexpr int kWideCap = kWinCap / 2;   // entries of C per window of wide slots
+static_assert(kWideCap >= kSubCols, "a window holds any single sub-block");
 
 // A window of a row, as k_win_plan lists it.
 struct alignas(64) WinRecord {
@@ -58,24 +66,29 @@ struct alignas(64) WinRecord {
   int32_t wb, we;  // sub-blocks [wb, we) of the row
   int32_t w0;      // first column (of a stacked batch: in the stacked product)
   int32_t row;
+  int32_t wide;    // kModeF32C: the row's entries need their term counts (wide slots, at most kWideCap of them)
 };
 static_assert(sizeof(WinRecord) == 64, "a record is four 16-byte pieces");
 
 // A chunk's segments (the parts of its A entries' B rows in the window), as lists of those with at
 // least one whole group of 32 products and of those with a remainder of fewer than 32, numbered
 // consecutively in each list.
+template <typename V>
 struct SegmentList {
-  double av[kChunk];      // a_ik
+  V av[kChunk];           // a_ik
   uint32_t bs[kChunk];    // start in B less the number of the segment's first product
   int32_t end[kChunk];    // end of its numbers (groups, or products)
 };
 
+template <typename V>
 struct TeamSmem {
-  double vals[kWinCap];                 // sums by rank
+  // By rank. kModeF64: the sums. kModeF32C: arrays of kWinCap FP32 sums and compensations; wide: of
+  // kWideCap sums, compensations, sums of |p| and term counts.
+  double vals[kWinCap];
   uint32_t bits[2][kWinSpan * 32];      // bitmap words of this window and the next
   uint16_t pre[kWinSpan * 32];          // set bits before each word
   uint16_t col[kWinCap];                // columns by rank, from the window's first
-  SegmentList whole, rest;              // the chunk's segments
+  SegmentList<V> whole, rest;           // the chunk's segments
   WinRecord rec[kSlots];
   unsigned long long tot[kTeam];
   int32_t have[kSlots];                 // a record follows in this slot
@@ -90,13 +103,16 @@ __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;
 
 // The windows of every row of perm[0, count): a warp per row takes the row's sub-blocks 64 at a time
 // (two counts per lane) and cuts windows greedily; a window ends at merge_cap entries (one sub-block may
-// have more), at kWinSpan sub-blocks, or with those 64.
+// have more), at kWinSpan sub-blocks, or with those 64. kModeF32C (negflag given: whether A or B has a
+// negative value): an entry of a row whose products are all non-negative and few enough is within the
+// bound without counting its terms (f32c_within_count); the other rows' windows have wide slots.
 __global__ void __launch_bounds__(256) k_win_plan(DevCsr A, const int32_t* __restrict__ perm, int64_t count,
                                                   const int32_t* __restrict__ win_slot, int64_t nslots,
                                                   const uint16_t* __restrict__ subcnt, int64_t nsub, int32_t merge_cap,
                                                   const int64_t* __restrict__ c_off, const int64_t* __restrict__ woff,
                                                   const int32_t* __restrict__ abase,
                                                   const int32_t* __restrict__ awidth, int64_t width_all,
+                                                  const int32_t* __restrict__ negflag,
                                                   WinRecord* __restrict__ wins, int64_t cap, int32_t* n_wins,
                                                   uint32_t* err) {
   const int lane = threadIdx.x & 31;
@@ -116,6 +132,8 @@ __global__ void __launch_bounds__(256) k_win_plan(DevCsr A, const int32_t* __res
     w.a0 = A.rp[i];
     w.na = static_cast<int32_t>(A.rp[i + 1] - w.a0);
     w.row = i;
+    w.wide = negflag && (*negflag != 0 || !f32c_within_count(w.na < (1 << 30) ? w.na : (1 << 30)));
+    const int32_t most = w.wide ? kWideCap : kWinCap, row_cap = merge_cap < most ? merge_cap : most;
     const int64_t out0 = c_off[i], room = c_off[i + 1] - out0, bits0 = woff[slot];
     int64_t at = 0;
     for (int pass = 0; pass < 2; ++pass) {
@@ -134,8 +152,8 @@ __global__ void __launch_bounds__(256) k_win_plan(DevCsr A, const int32_t* __res
           const int32_t base = s == 0 ? 0 : __shfl_sync(kFull, s <= 32 ? sa : sb, (s - 1) & 31);
           // the sub-blocks from s on that fit the window (the first always does)
           const uint64_t fit =
-              both(lane == s || (sa - base <= merge_cap && lane >= s && lane < s + kWinSpan),
-                   lane + 32 == s || (sb - base <= merge_cap && lane + 32 >= s && lane + 32 < s + kWinSpan)) & todo;
+              both(lane == s || (sa - base <= row_cap && lane >= s && lane < s + kWinSpan),
+                   lane + 32 == s || (sb - base <= row_cap && lane + 32 >= s && lane + 32 < s + kWinSpan)) & todo;
           const int e = 64 - __clzll(static_cast<long long>(fit));   // past the last non-empty one
           todo &= e == 64 ? 0ull : ~0ull << e;
           w.cnt = __shfl_sync(kFull, e <= 32 ? sa : sb, (e - 1) & 31) - base;
@@ -146,7 +164,7 @@ __global__ void __launch_bounds__(256) k_win_plan(DevCsr A, const int32_t* __res
             w.out = out0 + carry + base;
             w.bits = bits0 + int64_t(w.wb) * 32;
             w.cnts = int64_t(slot) * nsub + w.wb;
-            if (w.cnt > kWinCap || carry + base + w.cnt > room) {   // never writes past the rank array or the row
+            if (w.cnt > most || carry + base + w.cnt > room) {   // never writes past the rank array or the row
               set_error(err, kErrWindowPlan);
               w.cnt = w.na = 0;
             }
@@ -221,6 +239,7 @@ struct Window {
   const uint16_t* pre;
   double* vals;
   uint16_t* col;
+  bool wide, neg;   // kModeF32C
 };
 
 // Segments of a list of n that end at or before x: the number of the one that owns x.
@@ -234,15 +253,37 @@ __device__ __forceinline__ int first_after(const int32_t* end, int n, int32_t x)
 }
 
 // kGroups products per lane: a * v at column c (want bit u: the lane's u-th takes part).
+template <typename V>
 struct Step {
   int32_t c[kGroups];
-  double a[kGroups], v[kGroups];
+  V a[kGroups], v[kGroups];
   unsigned want;
 };
 
+// Adds the product a * b into the slot of rank r.
+__device__ __forceinline__ void add_product(const Window& win, int r, double a, double b) { atomicAdd(win.vals + r, a * b); }
+
+// FP32: the error-free product ph + pl, and the sum's own rounding error (TwoSum) rebuilt from the value
+// the atomic returns, as the other compensated kernels do (Dot2 accumulated concurrently).
+__device__ __forceinline__ void add_product(const Window& win, int r, float a, float b) {
+  float* slot = reinterpret_cast<float*>(win.vals) + r;
+  const float ph = a * b;
+  const float pl = fmaf(a, b, -ph);
+  const float old = atomicAdd(slot, ph);
+  const float nw = old + ph;
+  const float bp = nw - old;
+  const float q = (old - (nw - bp)) + (ph - bp);
+  atomicAdd(slot + (win.wide ? kWideCap : kWinCap), q + pl);
+  if (win.wide) {
+    if (win.neg) atomicAdd(slot + 2 * kWideCap, fabsf(ph));
+    atomicAdd(reinterpret_cast<int*>(slot) + 3 * kWideCap, 1);
+  }
+}
+
 // A step's products into the window's sums. The ranks of all of them are looked up before the first is
 // added.
-__device__ __forceinline__ void add_step(const Window& win, const Step& st, bool& bad) {
+template <typename V>
+__device__ __forceinline__ void add_step(const Window& win, const Step<V>& st, bool& bad) {
   const auto& c = st.c;
   const auto& a = st.a;
   const auto& v = st.v;
@@ -267,15 +308,16 @@ __device__ __forceinline__ void add_step(const Window& win, const Step& st, bool
   for (int u = 0; u < kGroups; ++u)
     if (r[u] >= 0) {
       win.col[r[u]] = static_cast<uint16_t>(rel[u]);   // every product of the column stores the same
-      atomicAdd(win.vals + r[u], a[u] * v[u]);
+      add_product(win, r[u], a[u], v[u]);
     }
 }
 static_assert(kWinSpan * kSubCols <= 65536, "a window's columns fit 16 bits");
 
 // One step of the whole groups: groups [g, g + kGroups) of the list's `groups` in n segments.
-__device__ __forceinline__ void load_whole(const SegmentList& sl, int n, int32_t g, int32_t groups,
-                                           const int32_t* __restrict__ bcol, const double* __restrict__ bval,
-                                           Step& st) {
+template <typename V>
+__device__ __forceinline__ void load_whole(const SegmentList<V>& sl, int n, int32_t g, int32_t groups,
+                                           const int32_t* __restrict__ bcol, const V* __restrict__ bval,
+                                           Step<V>& st) {
   const int lane = threadIdx.x & 31;
   const int o = first_after(sl.end, n, g);
   // every segment has a group, so kGroups groups see at most kGroups segments
@@ -297,9 +339,10 @@ __device__ __forceinline__ void load_whole(const SegmentList& sl, int n, int32_t
 }
 
 // One step of the remainders: products [p, p + 32 * kGroups) of the list's `total` in n segments.
-__device__ __forceinline__ void load_rest(const SegmentList& sl, int n, int32_t p, int32_t total,
-                                          const int32_t* __restrict__ bcol, const double* __restrict__ bval,
-                                          Step& st) {
+template <typename V>
+__device__ __forceinline__ void load_rest(const SegmentList<V>& sl, int n, int32_t p, int32_t total,
+                                          const int32_t* __restrict__ bcol, const V* __restrict__ bval,
+                                          Step<V>& st) {
   const int lane = threadIdx.x & 31;
   int o = first_after(sl.end, n, p);
   int k[kGroups];
@@ -350,16 +393,21 @@ __device__ __forceinline__ uint32_t lower_bound_at(const int32_t* __restrict__ c
   return s;
 }
 
+// V: double (kModeF64) or float (kModeF32C; row_flag takes the rows with an entry over the bound).
+template <typename V>
 __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
     DevCsr A, DevCsr B, const WinRecord* __restrict__ wins, const int32_t* __restrict__ n_wins, int64_t wins_cap,
     int32_t* counter, const uint16_t* __restrict__ subcnt, int64_t nsub, const uint32_t* __restrict__ split,
-    int32_t* __restrict__ ccol, double* __restrict__ cval, const uint32_t* __restrict__ wbits, uint32_t* err) {
+    int32_t* __restrict__ ccol, V* __restrict__ cval, const uint32_t* __restrict__ wbits,
+    const int32_t* __restrict__ negflag, int32_t* row_flag, uint32_t* err) {
   extern __shared__ __align__(64) unsigned char win_smem[];
-  TeamSmem& sw = *reinterpret_cast<TeamSmem*>(win_smem);
+  TeamSmem<V>& sw = *reinterpret_cast<TeamSmem<V>*>(win_smem);
+  constexpr bool kF32 = sizeof(V) == 4;
+  const bool neg = kF32 && *negflag != 0;
   constexpr int kThreads = kTeam * 32;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const double* aval = static_cast<const double*>(A.val);
-  const double* bval = static_cast<const double*>(B.val);
+  const V* aval = static_cast<const V*>(A.val);
+  const V* bval = static_cast<const V*>(B.val);
   const int32_t n = static_cast<int32_t>(*n_wins < wins_cap ? *n_wins : wins_cap);
   bool bad = false;
   // What a window needs first is fetched while the one before is worked on: its record two windows
@@ -375,14 +423,14 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
     for (int t = threadIdx.x; t < pieces; t += kThreads) copy16(&sw.bits[buf][4 * t], wbits + r.bits + 4 * t);
   };
   int32_t k1 = -1, ca = 0, cc = 0;
-  double v1 = 0.0;
+  V v1 = 0;
   auto fetch_entries = [&](const WinRecord& r) {
     const int ns = r.we - r.wb;
     ca = lane < ns ? subcnt[r.cnts + lane] : 0;
     cc = lane + 32 < ns ? subcnt[r.cnts + lane + 32] : 0;
     const bool mine = static_cast<int>(threadIdx.x) < r.na;
     k1 = mine ? A.col[r.a0 + threadIdx.x] : -1;
-    v1 = mine ? aval[r.a0 + threadIdx.x] : 0.0;
+    v1 = mine ? aval[r.a0 + threadIdx.x] : V(0);
   };
   auto bound = [&](const WinRecord& r, int32_t k, int32_t b) -> uint32_t {
     if (split) return split[k * nsub + b];
@@ -450,13 +498,21 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
           *reinterpret_cast<uint2*>(&sw.pre[t * 32 + lane * 4]) = make_uint2(p0 | p1 << 16, p2 | p3 << 16);
       }
     }
-    for (int q = threadIdx.x; q < (cnt + 1) / 2; q += kThreads)
-      reinterpret_cast<double2*>(sw.vals)[q] = make_double2(0.0, 0.0);
+    const bool wide = kF32 && r.wide != 0;
+    if constexpr (kF32) {
+      const int arrays = wide ? 4 : 2, stride = (wide ? kWideCap : kWinCap) / 4;
+      for (int q = threadIdx.x; q < (cnt + 3) / 4; q += kThreads)
+        for (int w = 0; w < arrays; ++w)
+          reinterpret_cast<float4*>(sw.vals)[w * stride + q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      for (int q = threadIdx.x; q < (cnt + 1) / 2; q += kThreads)
+        reinterpret_cast<double2*>(sw.vals)[q] = make_double2(0.0, 0.0);
+    }
     // 2. products; inside a row of several chunks, the next chunk's entries and bounds are loaded ahead
-    const Window win{r.w0, static_cast<uint32_t>(ns) * kSubCols, sw.bits[buf], sw.pre, sw.vals, sw.col};
+    const Window win{r.w0, static_cast<uint32_t>(ns) * kSubCols, sw.bits[buf], sw.pre, sw.vals, sw.col, wide, neg};
     const int64_t a0 = r.a0;
     int32_t k2 = static_cast<int>(threadIdx.x) + kChunk < na ? A.col[a0 + threadIdx.x + kChunk] : -1;
-    double v2 = static_cast<int>(threadIdx.x) + kChunk < na ? aval[a0 + threadIdx.x + kChunk] : 0.0;
+    V v2 = static_cast<int>(threadIdx.x) + kChunk < na ? aval[a0 + threadIdx.x + kChunk] : V(0);
     for (int32_t c0 = 0; c0 == 0 || c0 < na; c0 += kChunk) {
       // one scan numbers the whole groups (20 bits), the remainders (16), and both lists' segments
       const uint32_t len = be - bs, nw = len >> 5, nr = len & 31;
@@ -493,7 +549,7 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
         v1 = v2;
         const int32_t q3 = c0 + 2 * kChunk + static_cast<int>(threadIdx.x);
         k2 = q3 < na ? A.col[a0 + q3] : -1;
-        v2 = q3 < na ? aval[a0 + q3] : 0.0;
+        v2 = q3 < na ? aval[a0 + q3] : V(0);
       } else if (sw.have[slot1]) {
         fetch_bits(sw.rec[slot1], buf ^ 1);
         fetch_entries(sw.rec[slot1]);
@@ -502,15 +558,15 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
       const int32_t groups = static_cast<int32_t>(all & 0xfffff), rest = static_cast<int32_t>(all >> 20) & 0xffff;
       // the warps take the steps of both lists in turn: at most one step of each list is short
       const int wsteps = (groups + kGroups - 1) / kGroups, steps = wsteps + (rest + 32 * kGroups - 1) / (32 * kGroups);
-      auto load = [&](int q, Step& st) {
+      auto load = [&](int q, Step<V>& st) {
         if (q < wsteps) load_whole(sw.whole, static_cast<int>(all >> 36) & 0xfff, kGroups * q, groups, B.col, bval, st);
         else load_rest(sw.rest, static_cast<int>(all >> 48), 32 * kGroups * (q - wsteps), rest, B.col, bval, st);
       };
       if (wid < steps) {
-        Step cur;
+        Step<V> cur;
         load(wid, cur);
         for (int q = wid + kTeam; q < steps; q += kTeam) {   // a step's loads are under way while the last is added
-          Step ahead;
+          Step<V> ahead;
           load(q, ahead);
           add_step(win, cur, bad);
           cur = ahead;
@@ -537,10 +593,22 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
     {
       const int64_t out = r.out;
       const int32_t first = r.wb * kSubCols;
+      bool missed = false;
       for (int q = threadIdx.x; q < cnt; q += kThreads) {
         ccol[out + q] = first + sw.col[q];
-        cval[out + q] = sw.vals[q];
+        if constexpr (kF32) {
+          const float* f = reinterpret_cast<const float*>(sw.vals) + q;
+          const float res = f[0] + f[wide ? kWideCap : kWinCap];
+          cval[out + q] = res;
+          if (wide) {
+            const int t = __float_as_int(f[3 * kWideCap]);
+            missed |= neg ? !f32c_within_bound(res, f[2 * kWideCap], t) : !f32c_within_count(t);
+          }
+        } else {
+          cval[out + q] = sw.vals[q];
+        }
       }
+      if (missed) row_flag[r.row] = 1;
     }
     copies_done();
     slot = slot1;
@@ -552,10 +620,11 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
 
 }  // namespace
 
-int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merge_cap, int64_t* cap) {
+int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merge_cap, int f32c, int64_t* cap) {
   // a window ends by its span or the end of a run of 64 sub-blocks, or it and the next hold more than
   // merge_cap entries together; and it holds at least one sub-block
-  const int64_t m = merge_cap < 1 ? 1 : (merge_cap < kWinCap ? merge_cap : kWinCap);
+  const int64_t most = f32c ? kWideCap : kWinCap;
+  const int64_t m = merge_cap < 1 ? 1 : (merge_cap < most ? merge_cap : most);
   const int64_t by_entries = 2 * (entries / m + 1) + rows * ((nsub + 63) / 64 + nsub / kWinSpan + 1);
   *cap = by_entries < rows * nsub ? by_entries : rows * nsub;
   return *cap * static_cast<int64_t>(sizeof(WinRecord));
@@ -563,15 +632,15 @@ int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merg
 
 int launch_win_plan(const DevCsr& A, const int32_t* perm, int64_t count, const int32_t* win_slot, int64_t nslots,
                     const uint16_t* subcnt, int64_t nsub, int32_t merge_cap, const int64_t* c_off, const int64_t* woff,
-                    const int32_t* abase, const int32_t* awidth, int64_t width, void* wins, int64_t cap,
-                    int32_t* n_wins, int num_sms, uint32_t* err, cudaStream_t s) {
+                    const int32_t* abase, const int32_t* awidth, int64_t width, const int32_t* negflag, void* wins,
+                    int64_t cap, int32_t* n_wins, int num_sms, uint32_t* err, cudaStream_t s) {
   if (count <= 0) return 0;
   cudaMemsetAsync(n_wins, 0, sizeof(int32_t), s);
   int64_t g = (count + 7) / 8;
   if (g > int64_t(num_sms) * 8) g = int64_t(num_sms) * 8;
   k_win_plan<<<static_cast<unsigned>(g), 256, 0, s>>>(A, perm, count, win_slot, nslots, subcnt, nsub,
                                                       merge_cap < kWinCap ? merge_cap : kWinCap, c_off, woff, abase,
-                                                      awidth, width, static_cast<WinRecord*>(wins), cap, n_wins, err);
+                                                      awidth, width, negflag, static_cast<WinRecord*>(wins), cap, n_wins, err);
   return 1;
 }
 
@@ -585,14 +654,19 @@ int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint3
 
 int launch_num_winteam(const DevCsr& A, const DevCsr& B, const void* wins, const int32_t* n_wins, int64_t wins_cap,
                        int32_t* counter, const uint16_t* subcnt, int64_t nsub, const uint32_t* split, int32_t* ccol,
-                       double* cval, const uint32_t* wbits, int num_sms, uint32_t* err, cudaStream_t s) {
-  constexpr int smem = static_cast<int>(sizeof(TeamSmem));
-  static_assert(kTeamBlocks * (smem + 1024) <= 228 * 1024, "blocks per SM");
-  cudaFuncSetAttribute(k_num_winteam, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                       void* cval, const uint32_t* wbits, const int32_t* negflag, int32_t* row_flag, int num_sms,
+                       uint32_t* err, cudaStream_t s) {
   const unsigned grid = static_cast<unsigned>(num_sms * kTeamBlocks);
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
-  k_num_winteam<<<grid, kTeam * 32, smem, s>>>(A, B, static_cast<const WinRecord*>(wins), n_wins, wins_cap, counter,
-                                               subcnt, nsub, split, ccol, cval, wbits, err);
+  auto go = [&](auto kernel, auto* out) {
+    constexpr int smem = static_cast<int>(sizeof(TeamSmem<std::remove_pointer_t<decltype(out)>>));
+    static_assert(kTeamBlocks * (smem + 1024) <= 228 * 1024, "blocks per SM");
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    kernel<<<grid, kTeam * 32, smem, s>>>(A, B, static_cast<const WinRecord*>(wins), n_wins, wins_cap, counter, subcnt,
+                                          nsub, split, ccol, out, wbits, negflag, row_flag, err);
+  };
+  if (negflag) go(k_num_winteam<float>, static_cast<float*>(cval));
+  else go(k_num_winteam<double>, static_cast<double*>(cval));
   return 1;
 }
 

@@ -167,17 +167,19 @@ int launch_rerun_dense(const DevCsr& A, const DevCsr& B, const int32_t* rows, in
                        int64_t group_rows, int num_sms, uint32_t* err, cudaStream_t s);
 
 // ---- windowed rows of plans that store all their bitmaps (k_winteam.cu). The list of windows (its
-// bytes, and room for *cap windows; their number at *n_wins), built once per plan; the split table of
-// B by sub-blocks (B.rows * nsub + 1 words); the numeric pass itself, columns included.
-int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merge_cap, int64_t* cap);
+// bytes, and room for *cap windows; their number at *n_wins), built once per plan (kModeF32C: for each
+// numeric pass, as it depends on the values' signs); the split table of B by sub-blocks (B.rows * nsub +
+// 1 words); the numeric pass itself, columns included. negflag and row_flag: kModeF32C, else null.
+int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merge_cap, int f32c, int64_t* cap);
 int launch_win_plan(const DevCsr& A, const int32_t* perm, int64_t count, const int32_t* win_slot, int64_t nslots,
                     const uint16_t* subcnt, int64_t nsub, int32_t merge_cap, const int64_t* c_off, const int64_t* woff,
-                    const int32_t* abase, const int32_t* awidth, int64_t width, void* wins, int64_t cap,
-                    int32_t* n_wins, int num_sms, uint32_t* err, cudaStream_t s);
+                    const int32_t* abase, const int32_t* awidth, int64_t width, const int32_t* negflag, void* wins,
+                    int64_t cap, int32_t* n_wins, int num_sms, uint32_t* err, cudaStream_t s);
 int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint32_t* split, cudaStream_t s);
 int launch_num_winteam(const DevCsr& A, const DevCsr& B, const void* wins, const int32_t* n_wins, int64_t wins_cap,
                        int32_t* counter, const uint16_t* subcnt, int64_t nsub, const uint32_t* split, int32_t* ccol,
-                       double* cval, const uint32_t* wbits, int num_sms, uint32_t* err, cudaStream_t s);
+                       void* cval, const uint32_t* wbits, const int32_t* negflag, int32_t* row_flag, int num_sms,
+                       uint32_t* err, cudaStream_t s);
 
 int64_t split_table_bytes(int64_t brows, int64_t nblocks);
 int launch_bsplit(const DevCsr& B, int64_t nblocks, const int32_t* bbase, int32_t* split, cudaStream_t s);

@@ -355,9 +355,9 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
     const int64_t budget = (int64_t(p->opts.window_cols_max_mb > 0 ? p->opts.window_cols_max_mb : 0) << 20) / 4;
     const int64_t need = nwin * p->nblocks * kBlockWords;
     p->wcap = need < budget ? need : budget;
-    // all of them stored: the warp-per-window numeric pass, which plans by sub-blocks and numbers
+    // all of them stored: the numeric pass over a list of windows, which plans by sub-blocks and numbers
     // B's entries with 32 bits
-    p->sub = p->prec == SPGEMM_F64 && p->opts.fp64_accumulate == 0 && need <= budget && p->width <= kSymWinBits &&
+    p->sub = (p->prec != SPGEMM_F64 || p->opts.fp64_accumulate == 0) && need <= budget && p->width <= kSymWinBits &&
              B->nnz <= 0x7fffffffLL;
     if (p->sub) p->nblocks = (p->width + kSubCols - 1) / kSubCols;
     p->blockcnt = ws_get<uint16_t>(p, nwin * p->nblocks, &st);
@@ -519,7 +519,8 @@ int64_t window_list_cap(const spgemm_plan_s* p, int64_t nwin) {
 int64_t window_list_bytes(const spgemm_plan_s* p, int64_t nwin, int64_t* cap) {
   unsigned long long entries = 0;
   for (int c = kNumWin0; c <= kNumWin3; ++c) entries += p->cls_sums[c][2];
-  return win_list_bytes(nwin, static_cast<int64_t>(entries), p->nblocks, p->opts.window_hash_fill, cap);
+  return win_list_bytes(nwin, static_cast<int64_t>(entries), p->nblocks, p->opts.window_hash_fill,
+                        p->prec == SPGEMM_F32_COMPENSATED, cap);
 }
 
 int64_t split_sub_bytes(const spgemm_plan_s* p) { return p->B.rows * p->nblocks * int64_t(sizeof(uint32_t)); }
@@ -539,17 +540,21 @@ int numeric_windows(spgemm_plan_s* p, const int32_t* perm, int64_t nwin, int64_t
       if (p->split_sub) nl += launch_bsplit_sub(p->B, p->nblocks, p->bbase, p->split_sub, s);
     }
   }
-  if (!p->wins) {
+  const bool f32c = p->prec == SPGEMM_F32_COMPENSATED;
+  const int32_t* neg = f32c ? p->counters + 8 : nullptr;
+  const bool listed = p->wins != nullptr;
+  if (!listed) {
     const int64_t bytes = window_list_bytes(p, nwin, &p->wins_cap);
     p->wins = p->ws.get(static_cast<size_t>(bytes));
     if (!p->wins) return -1;
-    nl += launch_win_plan(p->A, perm, nwin, p->win_slot, nslots, p->blockcnt, p->nblocks, p->opts.window_hash_fill,
-                          p->c_off, p->woff, p->abase, p->awidth, p->width, p->wins, p->wins_cap, p->counters + 9,
-                          p->num_sms, &p->summary->err, s);
   }
+  if (!listed || f32c)
+    nl += launch_win_plan(p->A, perm, nwin, p->win_slot, nslots, p->blockcnt, p->nblocks, p->opts.window_hash_fill,
+                          p->c_off, p->woff, p->abase, p->awidth, p->width, neg, p->wins, p->wins_cap,
+                          p->counters + 9, p->num_sms, &p->summary->err, s);
   return nl + launch_num_winteam(p->A, p->B, p->wins, p->counters + 9, p->wins_cap, p->counters + 1, p->blockcnt,
-                                 p->nblocks, p->split_sub, C->col, static_cast<double*>(C->val), p->wbits, p->num_sms,
-                                 &p->summary->err, s);
+                                 p->nblocks, p->split_sub, C->col, C->val, p->wbits, neg, f32c ? p->rerun_flag : nullptr,
+                                 p->num_sms, &p->summary->err, s);
 }
 
 }  // namespace
