@@ -187,9 +187,81 @@ __global__ void __launch_bounds__(NT) k_sym_block(DevCsr A, DevCsr B, const int3
   }
 }
 
+// Bitmap words of the windowed pass with six and with three blocks on an SM.
+constexpr int kSymWinWords6 = 1 << 13;
+constexpr int kSymWinWords3 = 1 << 14;
+
+// Block rows in a column space of at most kSymBitmapCols: one bit per column in shared memory. A product
+// whose atomic finds its bit clear counts, so there is no counting pass; the products of a row of one
+// step per warp (all of them, unless the width itself is below block_max) stay in registers and clear
+// their words afterwards. The hash table it replaces cleared 8,192 slots a row and probed: 20,000^2
+// uniform (d = 2e-3, 19,000 rows of 1,600 products) 231 -> 145 us.
+constexpr int kSymBitmapCols = kSymWinWords6 * 32;
+template <int NT, int Blocks>
+__global__ void __launch_bounds__(NT, Blocks) k_sym_bitmap(DevCsr A, DevCsr B, int bitmap_words,
+                                                           const int32_t* __restrict__ perm, int64_t count,
+                                                           int32_t* __restrict__ nnz_row,
+                                                           const int32_t* __restrict__ abase, uint32_t* err) {
+  extern __shared__ uint32_t bm[];  // bitmap_words
+  __shared__ int32_t s_excl[NT + 1];
+  __shared__ int64_t s_bs[NT];
+  __shared__ long long s_scan64[33];
+  __shared__ int32_t s_ctl[2];
+  __shared__ int32_t s_cnt[2];
+  constexpr int kHold = 8;
+  for (int t = threadIdx.x; t < bitmap_words; t += NT) bm[t] = 0u;
+  if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+  __syncthreads();
+  const uint32_t span = static_cast<uint32_t>(bitmap_words) * 32u;
+  int turn = 0;
+  for (int64_t r = blockIdx.x; r < count; r += gridDim.x) {
+    const int32_t i = perm[r];
+    const int64_t a0 = A.rp[i];
+    const int64_t na = A.rp[i + 1] - a0;
+    const int32_t cb = abase ? abase[i] : 0;
+    uint32_t held[kHold];
+    int cnt = 0, steps = 0;
+    bool outside = false;
+    block_range_for_each_product<NT, kHold>(A, B, a0, na, s_excl, s_bs, s_scan64, s_ctl, [&](const int64_t (&j)[kHold]) {
+#pragma unroll
+      for (int u = 0; u < kHold; ++u) held[u] = j[u] >= 0 ? static_cast<uint32_t>(B.col[j[u]] - cb) : 0xffffffffu;
+#pragma unroll
+      for (int u = 0; u < kHold; ++u) {
+        if (held[u] < span) {
+          const uint32_t bit = 1u << (held[u] & 31);
+          cnt += (atomicOr(&bm[held[u] >> 5], bit) & bit) == 0u;
+        } else {
+          outside |= j[u] >= 0;
+        }
+      }
+      ++steps;
+    });
+    if (outside) set_error(err, kErrCount);
+    // (the enumeration ends with a barrier: every product of the row is marked)
+    const bool few = na <= NT && s_ctl[1] <= NT * kHold;
+    if (few) {
+      if (steps > 0)
+#pragma unroll
+        for (int u = 0; u < kHold; ++u)
+          if (held[u] < span) bm[held[u] >> 5] = 0u;
+    } else {
+      for (int t = threadIdx.x; t < bitmap_words; t += NT) bm[t] = 0u;
+    }
+    cnt = warp_sum(cnt);
+    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&s_cnt[turn], cnt);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      nnz_row[i] = s_cnt[turn];
+      s_cnt[turn] = 0;
+    }
+    turn ^= 1;
+  }
+}
+
 // Windowed symbolic pass, one row per block at a time (rows handed out by an atomic
 // counter, heaviest class first).
-__global__ void __launch_bounds__(kSymWinThreads, 1) k_sym_window(DevCsr A, DevCsr B,
+template <int NT, int Blocks>
+__global__ void __launch_bounds__(NT, Blocks) k_sym_window(DevCsr A, DevCsr B, int bitmap_words,
                                                                const int32_t* __restrict__ perm,
                                                                int64_t count, int32_t* counter,
                                                                int32_t* __restrict__ nnz_row,
@@ -201,18 +273,18 @@ __global__ void __launch_bounds__(kSymWinThreads, 1) k_sym_window(DevCsr A, DevC
                                                                int64_t width_all, uint32_t* __restrict__ wbits,
                                                                int64_t wcap, unsigned long long* wcur,
                                                                int64_t* __restrict__ woff, uint32_t* err) {
-  extern __shared__ uint32_t bm[];  // kSymWinBits / 32 words
-  __shared__ int32_t s_excl[kSymWinThreads + 1];
-  __shared__ int64_t s_bs[kSymWinThreads];
+  extern __shared__ uint32_t bm[];  // bitmap_words
+  __shared__ int32_t s_excl[NT + 1];
+  __shared__ int64_t s_bs[NT];
   __shared__ long long s_scan64[33];
   __shared__ int32_t s_ctl[2];
   __shared__ int32_t s_idx;
   __shared__ unsigned long long s_total;
   __shared__ long long s_woff;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  constexpr int kWarps = kSymWinThreads / 32;
+  constexpr int kWarps = NT / 32;
   // the bitmap is cleared once here; every window's counting pass leaves it clear again
-  for (int t = threadIdx.x; t < kSymWinBits / 32; t += kSymWinThreads) bm[t] = 0u;
+  for (int t = threadIdx.x; t < bitmap_words; t += NT) bm[t] = 0u;
   if (threadIdx.x == 0) {
     s_idx = atomicAdd(counter, 1);
     s_total = 0;
@@ -251,7 +323,7 @@ __global__ void __launch_bounds__(kSymWinThreads, 1) k_sym_window(DevCsr A, DevC
         const uint32_t span = static_cast<uint32_t>(wend - w0);
         const int32_t w0i = static_cast<int32_t>(w0);
         bool outside = false;
-        block_range_for_each_product<kSymWinThreads, 8>(
+        block_range_for_each_product<NT, 8>(
             A, B, a0, na, s_excl, s_bs, s_scan64, s_ctl, [&](const int64_t (&j)[8]) {
               int32_t c[8];
 #pragma unroll
@@ -372,12 +444,17 @@ int launch_sym_warp(int log2S, const DevCsr& A, const DevCsr& B, const int32_t* 
   return 1;
 }
 
-int launch_sym_block(int log2S, const DevCsr& A, const DevCsr& B, const int32_t* perm,
-                      int64_t count, int32_t* nnz_row, uint32_t* err, int num_sms, cudaStream_t s) {
+int launch_sym_block(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count, int32_t* nnz_row,
+                     const int32_t* abase, int64_t width, uint32_t* err, int num_sms, cudaStream_t s) {
   if (count <= 0) return 0;
-  const size_t sm = size_t(4) << log2S;
-  if (log2S == 13) {
-    k_sym_block<13, 512><<<grid_rows(count, 1, num_sms * 8), 512, sm, s>>>(A, B, perm, count, nnz_row, err);
+  if (width <= kSymBitmapCols) {
+    const int words = static_cast<int>((width + 31) / 32);
+    k_sym_bitmap<256, 6><<<grid_rows(count, 1, num_sms * 6), 256, 4 * words, s>>>(A, B, words, perm, count, nnz_row,
+                                                                                abase, err);
+  } else {
+    constexpr int kLog2 = 13;
+    k_sym_block<kLog2, 512><<<grid_rows(count, 1, num_sms * 8), 512, size_t(4) << kLog2, s>>>(A, B, perm, count,
+                                                                                             nnz_row, err);
   }
   return 1;
 }
@@ -386,15 +463,29 @@ int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int
                        int32_t* counter, int32_t* nnz_row, int32_t* win_slot, uint16_t* blockcnt,
                        int64_t nblocks, int sub, int32_t* cursor, const int32_t* abase, const int32_t* awidth,
                        int64_t width, uint32_t* wbits, int64_t wcap, unsigned long long* wcur, int64_t* woff,
-                       int num_sms, uint32_t* err, cudaStream_t s) {
+                       int64_t total_products, int64_t max_row_products, int num_sms, uint32_t* err,
+                       cudaStream_t s) {
   if (count <= 0) return 0;
-  const size_t sm = size_t(kSymWinBits / 32) * 4;
-  cudaFuncSetAttribute(k_sym_window, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
-  const int64_t g = count < num_sms ? count : num_sms;
-  k_sym_window<<<static_cast<unsigned>(g), kSymWinThreads, sm, s>>>(A, B, perm, count, counter, nnz_row,
-                                                                 win_slot, blockcnt, nblocks, sub, cursor,
-                                                                 abase, awidth, width, wbits, wcap, wcur, woff, err);
+  const int64_t cols = width < kSymWinBits ? width : kSymWinBits;
+  const int words = static_cast<int>((cols + kBlockCols - 1) / kBlockCols * kBlockWords);
+  auto go = [&](auto kernel, int threads, int blocks) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * words);
+    const int64_t g = count < int64_t(num_sms) * blocks ? count : int64_t(num_sms) * blocks;
+    kernel<<<static_cast<unsigned>(g), threads, 4 * words, s>>>(A, B, words, perm, count, counter, nnz_row, win_slot,
+                                                                blockcnt, nblocks, sub, cursor, abase, awidth, width,
+                                                                wbits, wcap, wcur, woff, err);
+  };
+  // The kernel waits for memory and at its barriers more than on anything else, so as many rows as the
+  // bitmaps leave room for are under way per SM. Measured, ms (R-MAT 2^17 with bitmaps of 16 KB, 30,000^2
+  // uniform, 4 KB; R-MAT 2^19, 64 KB): one block of 1,024 threads 2.82, 1.95; 19.7. Two of 512: 2.02,
+  // 1.50; 13.9. Three of 512: 1.79, 1.43; 12.4. Six of 256: 1.58, 1.32. Eight of 256: 1.78, 1.28.
+  // A single row that outweighs an SM's share of the products keeps the larger block, as its block
+  // finishes last.
+  const int64_t share = 2 * total_products / num_sms;
+  if (words <= kSymWinWords6 && max_row_products * 6 <= share) go(k_sym_window<256, 6>, 256, 6);
+  else if (words <= kSymWinWords3 && max_row_products * 3 <= share) go(k_sym_window<512, 3>, 512, 3);
+  else go(k_sym_window<kSymWinThreads, 1>, kSymWinThreads, 1);
   return 1;
 }
 

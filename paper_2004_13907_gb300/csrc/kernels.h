@@ -119,19 +119,21 @@ int launch_sym_micro(const DevCsr& A, const DevCsr& B, const int32_t* perm, int6
                      int32_t* nnz_row, int num_sms, cudaStream_t s);
 int launch_sym_warp(int log2S, const DevCsr& A, const DevCsr& B, const int32_t* perm,
                      int64_t count, int32_t* nnz_row, uint32_t* err, int num_sms, cudaStream_t s);
-int launch_sym_block(int log2S, const DevCsr& A, const DevCsr& B, const int32_t* perm,
-                      int64_t count, int32_t* nnz_row, uint32_t* err, int num_sms, cudaStream_t s);
+int launch_sym_block(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count, int32_t* nnz_row,
+                     const int32_t* abase, int64_t width, uint32_t* err, int num_sms, cudaStream_t s);
 // abase (per row of A, may be NULL = 0) and awidth (per row, may be NULL = width) give each
 // row's column space [abase[i], abase[i] + awidth[i]); blocks are counted from abase[i]. nblocks
 // (the block-count stride of a row) covers the widest row. wbits (may be NULL) receives, for each
 // row no wider than one symbolic window, its column bitmap (128 words per block of the row) at
 // word woff[slot], reserved from the cursor *wcur; -1 when the wcap words are used up or the row
-// is wider. sub: blockcnt counts sub-blocks of kSubCols columns (nblocks their number).
+// is wider. sub: blockcnt counts sub-blocks of kSubCols columns (nblocks their number). The products of
+// the whole plan and of its longest row choose the rows under way per SM.
 int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
                        int32_t* counter, int32_t* nnz_row, int32_t* win_slot, uint16_t* blockcnt,
                        int64_t nblocks, int sub, int32_t* cursor, const int32_t* abase, const int32_t* awidth,
                        int64_t width, uint32_t* wbits, int64_t wcap, unsigned long long* wcur, int64_t* woff,
-                       int num_sms, uint32_t* err, cudaStream_t s);
+                       int64_t total_products, int64_t max_row_products, int num_sms, uint32_t* err,
+                       cudaStream_t s);
 
 // ---- numeric kernels, FP64 (k_numeric.cu)
 int launch_num_tiny(int mode, const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,

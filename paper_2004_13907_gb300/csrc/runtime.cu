@@ -431,11 +431,12 @@ spgemm_status symbolic_run(spgemm_plan_s* p, cudaStream_t s) {
     if (p->wcur) cudaMemsetAsync(p->wcur, 0, sizeof(unsigned long long), s);
     nl = launch_sym_window(p->A, p->B, seg(kSymWin0), p->sym_off[kSymWin3 + 1] - p->sym_off[kSymWin0],
                            p->counters + 0, p->nnz_row, p->win_slot, p->blockcnt, p->nblocks, p->sub, p->cursor,
-                           p->abase, p->awidth, p->width, p->wbits, p->wcap, p->wcur, p->woff, p->num_sms, err,
-                           s);
+                           p->abase, p->awidth, p->width, p->wbits, p->wcap, p->wcur, p->woff,
+                           p->total_products, p->max_row_products, p->num_sms, err, s);
     stage_end(p, SPGEMM_STAGE_SYM_WINDOW, nl, s);
     stage_begin(p, SPGEMM_STAGE_SYM_BLOCK, s);
-    nl = launch_sym_block(13, p->A, p->B, seg(kSymBlock), cnt(kSymBlock), p->nnz_row, err, p->num_sms, s);
+    nl = launch_sym_block(p->A, p->B, seg(kSymBlock), cnt(kSymBlock), p->nnz_row, p->abase, p->width, err,
+                          p->num_sms, s);
     stage_end(p, SPGEMM_STAGE_SYM_BLOCK, nl, s);
     stage_begin(p, SPGEMM_STAGE_SYM_WARP, s);
     nl = launch_sym_warp(11, p->A, p->B, seg(kSymWarp3), cnt(kSymWarp3), p->nnz_row, err, p->num_sms, s);
