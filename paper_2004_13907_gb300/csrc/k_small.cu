@@ -34,6 +34,7 @@ constexpr int kSlots = 4;        // partial products per lane in one step (loads
 constexpr int kRunShared = 512;  // symbolic runs of up to this many rows keep their counts in shared memory
 constexpr int kSymWarpBytes = 4096;       // bitmap bytes per symbolic warp (all its row slots)
 constexpr int kNumSmemMax = 64 * 1024;   // numeric: 4 warps x (192 B x 32 + 10 B x 1,024) = 65,536 B at most
+constexpr double kFewEntries = 8.0, kFewProducts = 16.0;   // k_small_sym: Few, averages per row
 constexpr unsigned kFull = 0xffffffffu;
 enum : uint32_t { kSmallTooLong = 1u };   // summary->small_flags bit: a row needs the general path
 
@@ -287,6 +288,26 @@ __device__ __forceinline__ int rank_words(const uint32_t* bm, uint16_t* pre) {
   return carry;
 }
 
+// Ascending over the lanes.
+__device__ __forceinline__ uint32_t warp_sort(uint32_t key) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const uint32_t o = __shfl_xor_sync(kFull, key, j);
+      key = ((lane & j) == 0) == ((lane & k) == 0) ? min(key, o) : max(key, o);
+    }
+  }
+  return key;
+}
+
+// Lanes of a sorted run of keys that hold a key (not ~0) unlike the one before.
+__device__ __forceinline__ unsigned warp_heads(uint32_t key) {
+  const uint32_t before = __shfl_up_sync(kFull, key, 1);
+  return __ballot_sync(kFull, key != 0xffffffffu && ((threadIdx.x & 31) == 0 || before != key));
+}
+
 // Rank of column `col` in a row whose bits and word ranks are set.
 __device__ __forceinline__ int rank_of(const uint32_t* bm, const uint16_t* pre, int32_t col) {
   const int w = col >> 5;
@@ -296,7 +317,10 @@ __device__ __forceinline__ int rank_of(const uint32_t* bm, const uint16_t* pre, 
 // A warp takes G consecutive rows at a time (G = 1 to 4), each with a bitmap of its own, and
 // enumerates their partial products as one flat list, 32 entries of A at a time, so the memory
 // round trips of the group's rows overlap.
-template <int PER>
+// Few: four rows at a time and one bitmap. Their entries are read at once where they are at most 32, and
+// rows of at most 32 products together are counted by sorting (row, column) across the warp, without a
+// bitmap; the others take the bitmap one row after the other.
+template <int PER, bool Few>
 __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallCsr B, int32_t width, int check,
                                                               int64_t run, int G, int32_t* __restrict__ nnz_row,
                                                               int32_t* __restrict__ loc,
@@ -307,8 +331,9 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   __shared__ int32_t s_cnt[kRunShared];
   __shared__ bool s_last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t* bm0 = reinterpret_cast<uint32_t*>(small_smem) + static_cast<size_t>(wid) * G * 32 * PER;
-  for (int g = 0; g < G; ++g) Lanes<PER>::zero_all(bm0 + g * 32 * PER);
+  const int maps = Few ? 1 : G;
+  uint32_t* bm0 = reinterpret_cast<uint32_t*>(small_smem) + static_cast<size_t>(wid) * maps * 32 * PER;
+  for (int g = 0; g < maps; ++g) Lanes<PER>::zero_all(bm0 + g * 32 * PER);
   __syncwarp();
   const int64_t m = A.rows;
   const int64_t r0 = blockIdx.x * run < m ? blockIdx.x * run : m;
@@ -321,9 +346,14 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   // one says so at once, and the others, which look once per group (a load that the group's work hides),
   // stop there. Counting on to the end took 1.8 ms of a 30,000^2 product whose every row is too long.
   bool stop = false;
-  for (int64_t gs = r0 + wid * G; gs < r1 && !stop; gs += int64_t(kSymWarps) * G) {
-    const uint32_t flags = *reinterpret_cast<const volatile uint32_t*>(&sum->small_flags);
-    const int ng = r1 - gs < G ? static_cast<int>(r1 - gs) : G;
+  auto row_counted = [&](int64_t r, int cnt) {
+    if (lane == 0) {
+      nnz_row[r] = cnt;
+      if (run <= kRunShared) s_cnt[r - r0] = cnt;
+    }
+    max_cnt = cnt > max_cnt ? cnt : max_cnt;
+  };
+  auto bitmap_rows = [&](int64_t gs, int ng) {
     const RowGroup gr = group_rows(A, gs, ng, chk, bad);
     // lane g < ng: the first column of row gs + g's column space (a stacked batch's job)
     const int32_t cb_lane = A.cbase && lane < ng ? A.cbase[gs + lane] : 0;
@@ -358,12 +388,75 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
     for (int g = 0; g < 4; ++g) {
       if (g < ng) {
         const int cnt = warp_sum(cg[g]);
-        if (lane == 0) {
-          nnz_row[gs + g] = cnt;
-          if (run <= kRunShared) s_cnt[gs + g - r0] = cnt;
-        }
-        max_cnt = cnt > max_cnt ? cnt : max_cnt;
+        row_counted(gs + g, cnt);
       }
+    }
+    __syncwarp();
+  };
+  // rows [gs, gs + ng), at most four; false where they have more than 32 entries of A
+  auto sorted_rows = [&](int64_t gs, int ng) {
+    const RowGroup gr = group_rows(A, gs, ng, chk, bad);
+    if (gr.E > 32) return false;
+    const int32_t cb_lane = A.cbase && lane < ng ? A.cbase[gs + lane] : 0;
+    int g;
+    int64_t bs;
+    int32_t len;
+    double a;
+    group_chunk(A, B, gr, 0, chk, bad, g, bs, len, a);
+    prod += len;
+    unsigned long long tot = 0;   // products of each row, 16 bits (33: more than 32)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int s = __reduce_add_sync(kFull, g == t ? min(len, 33) : 0);
+      tot |= static_cast<unsigned long long>(min(s, 33)) << (16 * t);
+    }
+    auto of = [&](int t) { return static_cast<int>(tot >> (16 * t)) & 0xffff; };
+    for (int t = 0, e; t < ng; t = e) {
+      int sum = of(t);
+      for (e = t + 1; e < ng && sum + of(e) <= 32; ++e) sum += of(e);
+      uint32_t key = 0xffffffffu;
+      for_slots(g >= t && g < e ? len : 0, bs, a,
+                [&](const bool* ok, const int64_t* j, const int32_t*, const double*, const int* own) {
+                  int32_t c[kSlots];
+                  int go[kSlots];
+#pragma unroll
+                  for (int u = 0; u < kSlots; ++u) {
+                    c[u] = ok[u] ? B.col[j[u]] : -1;
+                    go[u] = __shfl_sync(kFull, g, own[u]);
+                    const int32_t cb = __shfl_sync(kFull, cb_lane, go[u]);
+                    c[u] = c[u] >= 0 ? c[u] - cb : -1;
+                  }
+#pragma unroll
+                  for (int u = 0; u < kSlots; ++u) {
+                    const bool in = c[u] >= 0 && c[u] < width;
+                    if (!in && ok[u] && chk) bad = true;   // a column outside its row's column space
+                    if (sum > 32) {
+                      if (in) atomicOr(&bm0[c[u] >> 5], 1u << (c[u] & 31));
+                    } else if (u == 0 && in) {
+                      key = static_cast<uint32_t>(go[0]) << 16 | static_cast<uint32_t>(c[0]);
+                    }
+                  }
+                });
+      if (sum > 32) {
+        __syncwarp();
+        row_counted(gs + t, warp_sum(count_clear<PER>(bm0)));
+        __syncwarp();
+      } else {
+        key = warp_sort(key);
+        const unsigned heads = warp_heads(key);
+        for (int q = t; q < e; ++q) row_counted(gs + q, __popc(heads & __ballot_sync(kFull, key >> 16 == static_cast<unsigned>(q))));
+      }
+    }
+    return true;
+  };
+  for (int64_t gs = r0 + wid * G; gs < r1 && !stop; gs += int64_t(kSymWarps) * G) {
+    const uint32_t flags = *reinterpret_cast<const volatile uint32_t*>(&sum->small_flags);
+    const int ng = r1 - gs < G ? static_cast<int>(r1 - gs) : G;
+    if constexpr (Few) {
+      if (!sorted_rows(gs, ng))
+        for (int t = 0; t < ng; ++t) bitmap_rows(gs + t, 1);
+    } else {
+      bitmap_rows(gs, ng);
     }
     if (max_cnt > kSmallCap) {
       if (lane == 0) atomicOr(&sum->small_flags, kSmallTooLong);
@@ -458,9 +551,11 @@ __device__ __forceinline__ void a_entry(const SmallCsr& A, const SmallCsr& B, in
 // enumerate their products twice. A product stores its column at its rank, so that columns leave by rank as
 // the values do. Bound by the instructions of a row and by few rows per warp; before, each lane walked
 // the bits of its words to write the row, a third of the kernel's instructions and scattered stores:
-// 10,000^2 uniform (d = 1e-3, the whole product) 78 -> 71 us.
+// 10,000^2 uniform (d = 1e-3, the whole product) 78 -> 71 us. A row of at most 32 products needs neither
+// bitmap nor ranks: one product per lane, sorted by column: 67,000 rows of 8 products on average, 100 ->
+// 50 us.
 template <int PER>
-__global__ void __launch_bounds__(kNumWarpsB * 32) k_small_num(SmallCsr A, SmallCsr B, int32_t width, int cap,
+__global__ void __launch_bounds__(kNumWarpsB * 32, PER <= 16 ? 9 : 7) k_small_num(SmallCsr A, SmallCsr B, int32_t width, int cap,
                                                                int64_t run,
                                                                const int32_t* __restrict__ nnz_row,
                                                                const int32_t* __restrict__ loc,
@@ -519,6 +614,30 @@ __global__ void __launch_bounds__(kNumWarpsB * 32) k_small_num(SmallCsr A, Small
           fv[u] = ok[u] ? av[u] * bv[j[u]] : 0.0;
         }
       });
+      if (ptot <= 32) {
+        // one product per lane: sorted by column (then by product), each run of a column summed by its
+        // first lane in product order; no bitmap
+        const uint32_t key = warp_sort(fc[0] >= 0 && fc[0] < width ? static_cast<uint32_t>(fc[0]) << 5 | lane : 0xffffffffu);
+        const uint32_t c = key == 0xffffffffu ? key : key >> 5;
+        const unsigned heads = warp_heads(c);
+        const double v0 = __shfl_sync(kFull, fv[0], key & 31);
+        double v = 0.0 + v0;
+        const bool head = heads >> lane & 1u;
+        for (int d = 1; d < 32; ++d) {
+          const uint32_t cd = __shfl_down_sync(kFull, c, d);
+          const bool more = head && lane + d < 32 && cd == c;
+          if (!__any_sync(kFull, more)) break;
+          const double vd = __shfl_down_sync(kFull, v0, d);
+          if (more) v += vd;
+        }
+        const int cnt = __popc(heads), r = __popc(heads & ((1u << lane) - 1u));
+        if (cnt != len) bad = true;
+        if (head && r < len) {
+          ccol[off + r] = static_cast<int32_t>(c);
+          cval[off + r] = v;
+        }
+        continue;
+      }
 #pragma unroll
       for (int u = 0; u < kSlots; ++u)
         if (fc[u] >= 0 && fc[u] < width) atomicOr(&bm[fc[u] >> 5], 1u << (fc[u] & 31));
@@ -593,8 +712,9 @@ int per_index(int per) { return __builtin_ctz(static_cast<unsigned>(per)); }
 
 template <int PER>
 void sym_launch(dim3 g, size_t smem, cudaStream_t s, const SmallCsr& A, const SmallCsr& B, int32_t width, int check,
-                int64_t run, int G, int32_t* nnz_row, int32_t* loc, int64_t* blk, Summary* sum, Summary* hsum) {
-  k_small_sym<PER><<<g, kSymWarps * 32, smem, s>>>(A, B, width, check, run, G, nnz_row, loc, blk, sum, hsum);
+                SmallGrid sg, int32_t* nnz_row, int32_t* loc, int64_t* blk, Summary* sum, Summary* hsum) {
+  const auto kernel = sg.few ? k_small_sym<PER, true> : k_small_sym<PER, false>;
+  kernel<<<g, kSymWarps * 32, smem, s>>>(A, B, width, check, sg.run, sg.groups, nnz_row, loc, blk, sum, hsum);
 }
 
 template <int PER>
@@ -612,14 +732,15 @@ __global__ void __launch_bounds__(256) k_small_offsets(const int32_t* __restrict
     c_off[i] = i < m ? blk[i / run] + loc[i] : blk[nblk];
 }
 
+template <bool Few>
 const void* sym_fn(int k) {
   switch (k) {
-    case 0: return reinterpret_cast<const void*>(k_small_sym<1>);
-    case 1: return reinterpret_cast<const void*>(k_small_sym<2>);
-    case 2: return reinterpret_cast<const void*>(k_small_sym<4>);
-    case 3: return reinterpret_cast<const void*>(k_small_sym<8>);
-    case 4: return reinterpret_cast<const void*>(k_small_sym<16>);
-    default: return reinterpret_cast<const void*>(k_small_sym<32>);
+    case 0: return reinterpret_cast<const void*>(k_small_sym<1, Few>);
+    case 1: return reinterpret_cast<const void*>(k_small_sym<2, Few>);
+    case 2: return reinterpret_cast<const void*>(k_small_sym<4, Few>);
+    case 3: return reinterpret_cast<const void*>(k_small_sym<8, Few>);
+    case 4: return reinterpret_cast<const void*>(k_small_sym<16, Few>);
+    default: return reinterpret_cast<const void*>(k_small_sym<32, Few>);
   }
 }
 
@@ -637,7 +758,7 @@ const void* num_fn(int k) {
 // Per device, once: the registers a thread of each kernel instance holds, and the numeric
 // kernels' dynamic shared memory limit raised to kNumSmemMax.
 struct SmallKernelInfo {
-  int sym_regs[kPerCount] = {}, num_regs[kPerCount] = {};
+  int sym_regs[2][kPerCount] = {}, num_regs[kPerCount] = {};
   bool ready = false;
 };
 
@@ -653,7 +774,11 @@ const SmallKernelInfo& small_info() {
   if (!k.ready) {
     for (int i = 0; i < kPerCount; ++i) {
       cudaFuncAttributes fa{};
-      k.sym_regs[i] = cudaFuncGetAttributes(&fa, sym_fn(i)) == cudaSuccess && fa.numRegs > 0 ? fa.numRegs : 64;
+      for (int few = 0; few < 2; ++few)
+        k.sym_regs[few][i] = cudaFuncGetAttributes(&fa, few ? sym_fn<true>(i) : sym_fn<false>(i)) == cudaSuccess &&
+                                     fa.numRegs > 0
+                                 ? fa.numRegs
+                                 : 64;
       k.num_regs[i] = cudaFuncGetAttributes(&fa, num_fn(i)) == cudaSuccess && fa.numRegs > 0 ? fa.numRegs : 64;
       cudaFuncSetAttribute(num_fn(i), cudaFuncAttributeMaxDynamicSharedMemorySize, kNumSmemMax);
     }
@@ -696,17 +821,23 @@ size_t num_smem(int per, int cap) { return num_warp_bytes(per, cap) * kNumWarpsB
 
 bool small_path_fits(int64_t m, int64_t n) { return m <= kSmallMaxRows && n <= kSmallMaxCols && n > 0; }
 
-SmallGrid small_sym_grid(const SmallCsr& A, int64_t width, int num_sms) {
+SmallGrid small_sym_grid(const SmallCsr& A, const SmallCsr& B, int64_t width, int num_sms) {
   const int per = small_per(width);
-  const int G = small_groups(avg_row(A), static_cast<size_t>(128) * per, kSymWarpBytes);
-  const int regs = small_info().sym_regs[per_index(per)];
+  // Short rows four at a time, sorted across the warp, where there are enough of them for every warp of
+  // the chip; with fewer the four take longer than four warps (1,000^2, 4 entries a row: 64 us against
+  // 60; 32,000^2: 98 against 108, 1 entry a row 85 against 102; a batch of 67,000 rows: 36 against 61 in
+  // the kernel). The averages are those of the whole product: a longer row takes the bitmap.
+  const bool few = A.rows >= int64_t(num_sms) * 64 && avg_row(A) <= kFewEntries &&
+                   avg_row(A) * avg_row(B) <= kFewProducts;
+  const int G = few ? 4 : small_groups(avg_row(A), static_cast<size_t>(128) * per, kSymWarpBytes);
+  const int regs = small_info().sym_regs[few][per_index(per)];
   const int64_t m = A.rows;
-  const int64_t cap = int64_t(num_sms) * resident(regs, kSymWarps * 32, sym_smem(per, G), 8);
+  const int64_t cap = int64_t(num_sms) * resident(regs, kSymWarps * 32, sym_smem(per, few ? 1 : G), 8);
   int64_t g = (m + int64_t(kSymWarps) * G - 1) / (int64_t(kSymWarps) * G);
   g = g < cap ? g : cap;
   g = g > 0 ? g : 1;
   const int64_t run = (m + g - 1) / g;
-  return SmallGrid{(m + run - 1) / run, run, G};
+  return SmallGrid{(m + run - 1) / run, run, G, few};
 }
 
 int launch_small_symbolic(const SmallCsr& A, const SmallCsr& B, int64_t width, SmallGrid g, int check,
@@ -714,10 +845,9 @@ int launch_small_symbolic(const SmallCsr& A, const SmallCsr& B, int64_t width, S
                           cudaStream_t s) {
   const int per = small_per(width);
   const dim3 grid(static_cast<unsigned>(g.blocks));
-  const size_t smem = sym_smem(per, g.groups);
-  const int G = g.groups;
+  const size_t smem = sym_smem(per, g.few ? 1 : g.groups);
   const int32_t w = static_cast<int32_t>(width);
-#define SPG_SYM(P) sym_launch<P>(grid, smem, s, A, B, w, check, g.run, G, nnz_row, loc, blk, sum, hsum)
+#define SPG_SYM(P) sym_launch<P>(grid, smem, s, A, B, w, check, g, nnz_row, loc, blk, sum, hsum)
   switch (per) {
     case 1: SPG_SYM(1); break;
     case 2: SPG_SYM(2); break;

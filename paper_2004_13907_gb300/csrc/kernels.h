@@ -58,12 +58,13 @@ struct SmallCsr {
 };
 bool small_path_fits(int64_t m, int64_t n);
 // The symbolic kernel's grid: `blocks` blocks, each a contiguous run of `run` rows, its warps
-// taking `groups` rows at a time.
+// taking `groups` rows at a time (few: short rows, counted without a bitmap where they allow it).
 struct SmallGrid {
   int64_t blocks, run;
   int groups;
+  bool few;
 };
-SmallGrid small_sym_grid(const SmallCsr& A, int64_t width, int num_sms);
+SmallGrid small_sym_grid(const SmallCsr& A, const SmallCsr& B, int64_t width, int num_sms);
 // Symbolic pass, validation of A and B (when `check`) and the offsets of C's rows, in one kernel:
 // nnz_row[i], loc[i] (row i's offset within its block's run), blk[b] (run b's offset, b <= blocks,
 // blk[blocks] = nnz(C)), summary->total (nnz(C)), max_row (longest row of C), small_products,

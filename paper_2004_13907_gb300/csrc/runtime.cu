@@ -188,7 +188,7 @@ spgemm_status plan_small(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_
   spgemm_status st = SPGEMM_OK;
   const int64_t m = A->rows;
   auto r256 = [](int64_t b) { return static_cast<size_t>((b + 255) & ~int64_t(255)); };
-  p->small_grid = small_sym_grid(small_csr(*A), p->abase ? p->width : B->cols, p->num_sms);
+  p->small_grid = small_sym_grid(small_csr(*A), small_csr(*B), p->abase ? p->width : B->cols, p->num_sms);
   const size_t sum_bytes = r256(sizeof(Summary));
   const size_t blk_bytes = r256(8 * (p->small_grid.blocks + 1));
   const size_t row_bytes = r256(4 * m);
