@@ -491,7 +491,8 @@ __global__ void __launch_bounds__(256) k_num_warp(DevCsr A, DevCsr B, const int3
 // registers, so that four rows are in flight on an SM; the hash table and bitonic sort of
 // k_num_block are bound by the sort's shared-memory traffic instead. Both block classes, hash
 // and bitonic sort -> bitmaps: 20,000^2 uniform (19,400 rows of 1,540 entries) 3.83 -> 0.36 ms,
-// R-MAT 2^17 2.67 -> 0.46 ms, R-MAT 2^19 7.87 -> 1.19 ms.
+// R-MAT 2^17 2.67 -> 0.46 ms, R-MAT 2^19 7.87 -> 1.19 ms. Columns stored by the products (Direct): 20,000^2
+// 0.355 -> 0.30 ms.
 constexpr int kHeld = 8;   // products per thread held in registers
 constexpr int kStep = 4;   // products per thread in one step (loads in flight)
 constexpr int64_t kBitmapMaxWidth = int64_t(1) << 22;   // coarse words: 16 KB
@@ -617,7 +618,9 @@ __device__ __forceinline__ void add_held(double* slot, double held) {
   }
 }
 
-template <int NT, int Mode>
+// Direct: every word of the column space fits the table, and a column 16 bits, so that a product stores
+// its column at its rank and no pass walks the bits.
+template <int NT, int Mode, bool Direct>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
                                                      int64_t count, const int64_t* __restrict__ c_off,
                                                      int32_t* __restrict__ ccol, void* __restrict__ cval,
@@ -628,14 +631,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
   extern __shared__ double smem_f64[];
   __shared__ BitmapChunk<NT> ck;
   double* vals = smem_f64;                                          // [cap], by rank
-  int32_t* colbuf = reinterpret_cast<int32_t*>(vals + cap);         // [cap], the row's columns by rank
-  int32_t* gword = colbuf + cap;                                    // [cap], two levels: word number of a table word
-  uint32_t* fine = reinterpret_cast<uint32_t*>(gword + cap);        // [cap], the word table (zero between rows)
-  uint32_t* coarse = fine + cap;                                    // a bit per word (zero between rows)
-  const int coarse_all = bitmap_coarse_words(width_all, cap);
-  uint16_t* fpre = reinterpret_cast<uint16_t*>(coarse + coarse_all);   // [cap]
-  uint16_t* cpre = fpre + cap;                                         // [coarse_all]
-  for (int t = threadIdx.x; t < cap + coarse_all; t += NT) fine[t] = 0u;
+  const int table = Direct ? (static_cast<int>(width_all) + 31) >> 5 : cap;   // words of the word table
+  const int coarse_all = Direct ? 0 : bitmap_coarse_words(width_all, cap);
+  uint32_t* fine = reinterpret_cast<uint32_t*>(vals + cap);         // [table], the word table (zero between rows)
+  uint32_t* coarse = fine + table;                                  // a bit per word (zero between rows)
+  int32_t* gword = reinterpret_cast<int32_t*>(coarse + coarse_all); // [cap], two levels: word number of a table word
+  int32_t* colbuf = gword + cap;                                    // [cap], two levels: the columns by rank
+  uint16_t* fpre = reinterpret_cast<uint16_t*>(Direct ? gword : colbuf + cap);   // [table]
+  uint16_t* cpre = fpre + table;                                    // [coarse_all]
+  uint16_t* cols = cpre;                                            // [cap], Direct: the columns by rank
+  for (int t = threadIdx.x; t < table + coarse_all; t += NT) fine[t] = 0u;
   for (int64_t r = blockIdx.x; r < count; r += gridDim.x) {
     const int32_t i = perm[r];
     const int64_t a0 = A.rp[i];
@@ -645,7 +650,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
     const int32_t cb = abase ? abase[i] : 0;   // the row's columns are [cb, cb + width)
     const uint32_t width = static_cast<uint32_t>(awidth ? awidth[i] : width_all);
     const int words = static_cast<int>((width + 31) >> 5);
-    const bool direct = words <= cap;
+    const bool direct = Direct || words <= cap;   // (a narrower job of a batch may fit where the widest does not)
     if (Mode == kModeF32C && threadIdx.x == 0 && !f32c_hash_row_ok(negflag, na)) row_flag[i] = 1;
     __syncthreads();   // the previous row's clearing of the bitmaps
     // the table word of column rel (two levels), -1 past the table (a row counted otherwise)
@@ -733,7 +738,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
     // pass 3: the products by rank
     auto add = [&](int g, int bit, double p) {
       const int rk = fpre[g] + __popc(fine[g] & ((1u << bit) - 1u));
-      if (rk < n_out) add_held<Mode>(&vals[rk], p);
+      if (rk < n_out) {
+        if constexpr (Direct) cols[rk] = static_cast<uint16_t>(g * 32 + bit);   // every product of the column the same
+        add_held<Mode>(&vals[rk], p);
+      }
     };
     if (keep) {
 #pragma unroll
@@ -763,19 +771,23 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
       }
     }
     // the columns by rank, and the bitmaps cleared for the next row
-    for (int w = threadIdx.x; w < nwords; w += NT) {
-      uint32_t m = fine[w];
-      if (!m) continue;
-      const int col0 = 32 * (direct ? w : gword[w]);
-      for (int rk = fpre[w]; m; m &= m - 1, ++rk)
-        if (rk < n_out) colbuf[rk] = col0 + __ffs(m) - 1;
-      fine[w] = 0u;
+    if constexpr (Direct) {
+      for (int w = threadIdx.x; w < nwords; w += NT) fine[w] = 0u;
+    } else {
+      for (int w = threadIdx.x; w < nwords; w += NT) {
+        uint32_t m = fine[w];
+        if (!m) continue;
+        const int col0 = 32 * (direct ? w : gword[w]);
+        for (int rk = fpre[w]; m; m &= m - 1, ++rk)
+          if (rk < n_out) colbuf[rk] = col0 + __ffs(m) - 1;
+        fine[w] = 0u;
+      }
+      if (!direct)
+        for (int w = threadIdx.x; w < cwords; w += NT) coarse[w] = 0u;
+      __syncthreads();
     }
-    if (!direct)
-      for (int w = threadIdx.x; w < cwords; w += NT) coarse[w] = 0u;
-    __syncthreads();
     for (int t = threadIdx.x; t < n_out; t += NT) {
-      ccol[off + t] = colbuf[t];
+      ccol[off + t] = Direct ? static_cast<int32_t>(cols[t]) : colbuf[t];
       store_value<Mode>(cval, off + t, vals[t]);
     }
     if (bad) set_error(err, kErrCount);
@@ -905,13 +917,16 @@ int launch_num_block(int log2S, int mode, const DevCsr& A, const DevCsr& B, cons
   if (width <= kBitmapMaxWidth) {
     const int cap = log2S == 11 ? 1024 : (max_nnz <= 2048 ? 2048 : 4096);
     const int cw = bitmap_coarse_words(width, cap);
-    const size_t sm = size_t(cap) * (8 + 4 + 4 + 4 + 2) + size_t(cw) * 6;
+    const bool direct = cw == 0 && width <= 65536;
+    const size_t sm = direct ? size_t(cap) * (8 + 2) + size_t((width + 31) / 32) * (4 + 2)
+                             : size_t(cap) * (8 + 4 + 4 + 4 + 2) + size_t(cw) * 6;
     auto go = [&](auto kernel) {
       if (sm > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
       kernel<<<grid_rows(count, 1, num_sms * 16), 256, sm, s>>>(A, B, perm, count, c_off, ccol, cval, abase, awidth, width,
                                                                cap, row_flag, negflag, err);
     };
-    f32c ? go(k_num_bitmap<256, kModeF32C>) : go(k_num_bitmap<256, kModeF64>);
+    if (direct) f32c ? go(k_num_bitmap<256, kModeF32C, true>) : go(k_num_bitmap<256, kModeF64, true>);
+    else f32c ? go(k_num_bitmap<256, kModeF32C, false>) : go(k_num_bitmap<256, kModeF64, false>);
     return 1;
   }
   const size_t sm = (size_t(1) << log2S) * 12;
