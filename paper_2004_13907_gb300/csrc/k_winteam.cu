@@ -19,12 +19,14 @@
 // more of them in flight, a list of windows lets the next one's data be fetched ahead, a product stores
 // its column at its rank on the way, so no pass extracts the columns from the bitmap, and whole groups
 // of 32 products of one segment need no search per product. Both kernels -> this one: 30,000^2
-// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 5.06 ms, R-MAT 2^17 (1.09e9) 9.92 -> 6.39 ms, R-MAT 2^19
-// (7.85e9) 77.6 -> 58.5 ms.
+// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 4.58 ms, R-MAT 2^17 (1.09e9) 9.92 -> 6.30 ms, R-MAT 2^19
+// (7.85e9) 77.6 -> 57.5 ms. Of this, finding a product's segment by a bit per segment start instead of a
+// search of the segments' ends (k_num_winteam issued 146 instructions per 32 products): 5.06 -> 4.58,
+// 6.39 -> 6.30, 58.6 -> 57.5.
 //
 // FP32-compensated plans take the same kernel with FP32 sums and compensations in the eight bytes of a
 // slot (two FP32 atomics a product, separate arrays so that both spread over all banks): R-MAT 2^17
-// 7.93 -> 6.12 ms. A slot that also needs the sum of |p| and the term count takes sixteen bytes and its
+// 7.93 -> 5.73 ms. A slot that also needs the sum of |p| and the term count takes sixteen bytes and its
 // windows half the entries; with mixed signs (R-MAT 2^17 of 8 edges a vertex) 4.51 -> 3.50 ms.
 #include <type_traits>
 
@@ -36,8 +38,8 @@ namespace spg {
 namespace {
 
 // A window's size against the number of windows an SM works on at once (one per block; a block is idle
-// while its window's ranks are made, at its barriers and while it writes out). Measured, ms of the
-// numeric pass on the 30,000^2 uniform product (d = 5e-3), R-MAT 2^17 and R-MAT 2^19:
+// while its window's ranks are made, at its barriers and while it writes out). Measured with a search of
+// the segments' ends, ms of the numeric pass on the 30,000^2 uniform product (d = 5e-3), R-MAT 2^17 and R-MAT 2^19:
 //   4 warps, 2048 entries, 32 sub-blocks, 6 blocks per SM: 5.06, 6.39, 58.5 (taken)
 //   4 warps, 1536 entries, 7 blocks: 5.63, 6.62, 62.1;  1152 entries, 8 blocks: 5.82, 6.99, 66.7
 //   4 warps, 1920 entries, 64 sub-blocks, 5 blocks: 5.70, 6.85, 61.5
@@ -74,11 +76,18 @@ static_assert(sizeof(WinRecord) == 64, "a record is four 16-byte pieces");
 // least one whole group of 32 products and of those with a remainder of fewer than 32, numbered
 // consecutively in each list.
 template <typename V>
-struct SegmentList {
+struct WholeList {
   V av[kChunk];           // a_ik
-  uint32_t bs[kChunk];    // start in B less the number of the segment's first product
-  int32_t end[kChunk];    // end of its numbers (groups, or products)
+  uint32_t bs[kChunk];    // start in B less 32 times the number of the segment's first group
+  int32_t end[kChunk];    // end of its numbers
 };
+template <typename V>
+struct RestList {
+  V av[kChunk];
+  uint32_t bs[kChunk];         // start in B less the number of the segment's first product
+  uint32_t start[2][kChunk];   // bit per product: a segment starts there (this chunk's, and zeros for the next)
+  uint8_t first[kChunk];       // per 32 products: the first segment that starts among them. None has 32
+};                             // products, so one does
 
 template <typename V>
 struct TeamSmem {
@@ -88,7 +97,8 @@ struct TeamSmem {
   uint32_t bits[2][kWinSpan * 32];      // bitmap words of this window and the next
   uint16_t pre[kWinSpan * 32];          // set bits before each word
   uint16_t col[kWinCap];                // columns by rank, from the window's first
-  SegmentList<V> whole, rest;           // the chunk's segments
+  WholeList<V> whole;                   // the chunk's segments
+  RestList<V> rest;
   WinRecord rec[kSlots];
   unsigned long long tot[kTeam];
   int32_t have[kSlots];                 // a record follows in this slot
@@ -243,13 +253,14 @@ struct Window {
 };
 
 // Segments of a list of n that end at or before x: the number of the one that owns x.
-__device__ __forceinline__ int first_after(const int32_t* end, int n, int32_t x) {
-  int o = 0;
-  for (int q = 0; q < n; q += 32) {
-    const int t = q + static_cast<int>(threadIdx.x & 31);
-    o += __popc(__ballot_sync(kFull, t < n && end[t] <= x));
+// A warp asks for ascending x: `from` (a multiple of 32, at first 0) is where its last answer was.
+__device__ __forceinline__ int first_after(const int32_t* end, int n, int32_t x, int& from) {
+  for (;;) {
+    const int t = from + static_cast<int>(threadIdx.x & 31);
+    const int o = __popc(__ballot_sync(kFull, t < n && end[t] <= x));
+    if (o < 32) return from + o;
+    from += 32;
   }
-  return o;
 }
 
 // kGroups products per lane: a * v at column c (want bit u: the lane's u-th takes part).
@@ -315,11 +326,11 @@ static_assert(kWinSpan * kSubCols <= 65536, "a window's columns fit 16 bits");
 
 // One step of the whole groups: groups [g, g + kGroups) of the list's `groups` in n segments.
 template <typename V>
-__device__ __forceinline__ void load_whole(const SegmentList<V>& sl, int n, int32_t g, int32_t groups,
+__device__ __forceinline__ void load_whole(const WholeList<V>& sl, int n, int32_t g, int32_t groups,
                                            const int32_t* __restrict__ bcol, const V* __restrict__ bval,
-                                           Step<V>& st) {
+                                           Step<V>& st, int& from) {
   const int lane = threadIdx.x & 31;
-  const int o = first_after(sl.end, n, g);
+  const int o = first_after(sl.end, n, g, from);
   // every segment has a group, so kGroups groups see at most kGroups segments
   const int32_t e = sl.end[min(o + lane, n - 1)];
   uint32_t j[kGroups];
@@ -338,43 +349,22 @@ __device__ __forceinline__ void load_whole(const SegmentList<V>& sl, int n, int3
   st.want = g + kGroups <= groups ? (1u << kGroups) - 1u : (1u << (groups - g)) - 1u;
 }
 
-// One step of the remainders: products [p, p + 32 * kGroups) of the list's `total` in n segments.
+// One step of the remainders: products [p, p + 32 * kGroups) of the list's `total` (p a multiple of 32).
 template <typename V>
-__device__ __forceinline__ void load_rest(const SegmentList<V>& sl, int n, int32_t p, int32_t total,
+__device__ __forceinline__ void load_rest(const RestList<V>& sl, const uint32_t* start, int32_t p, int32_t total,
                                           const int32_t* __restrict__ bcol, const V* __restrict__ bval,
                                           Step<V>& st) {
   const int lane = threadIdx.x & 31;
-  int o = first_after(sl.end, n, p);
-  int k[kGroups];
-  const int32_t e = o + lane < n ? sl.end[o + lane] - p : 0x7fffffff;   // > 0: o owns p
-  if (__shfl_sync(kFull, e, 31) >= 32 * kGroups) {
-    // at most 32 segments end among these products: a lane's segment is the number of ends at or
-    // before its product
-#pragma unroll
-    for (int u = 0; u < kGroups; ++u) {
-      const unsigned m = __reduce_or_sync(kFull, (e >> 5) == u ? 1u << (e & 31) : 0u);
-      k[u] = o + __popc(m & (0xffffffffu >> (31 - lane)));
-      o += __popc(m);
-    }
-  } else {
-    // many short segments: at most 32 more end in each group
-#pragma unroll
-    for (int u = 0; u < kGroups; ++u) {
-      const int32_t x = o + lane < n ? sl.end[o + lane] - (p + 32 * u) : 0x7fffffff;
-      const unsigned m = __reduce_or_sync(kFull, x >= 0 && x < 32 ? 1u << x : 0u);
-      k[u] = o + __popc(m & (0xffffffffu >> (31 - lane)));
-      o += __popc(m);
-    }
-  }
   uint32_t j[kGroups];
   st.want = 0;
 #pragma unroll
   for (int u = 0; u < kGroups; ++u) {
     const int32_t x = p + 32 * u + lane;
     if (x < total) st.want |= 1u << u;
-    const int q = min(k[u], n - 1);
-    j[u] = sl.bs[q] + static_cast<uint32_t>(min(x, total - 1));   // a lane past the end takes the last product
-    st.a[u] = sl.av[q];
+    const int32_t y = min(x, total - 1);   // a lane past the end takes the last product
+    const int k = sl.first[y >> 5] + __popc(start[y >> 5] & (0xffffffffu >> (31 - (y & 31)))) - 1;
+    j[u] = sl.bs[k] + static_cast<uint32_t>(y);
+    st.a[u] = sl.av[k];
   }
 #pragma unroll
   for (int u = 0; u < kGroups; ++u) {
@@ -437,6 +427,7 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
     return lower_bound_at(B.col, static_cast<uint32_t>(B.rp[k]), static_cast<uint32_t>(B.rp[k + 1]),
                           int64_t(r.w0) + int64_t(b - r.wb) * kSubCols);
   };
+  sw.rest.start[0][threadIdx.x] = 0u;
   int32_t next = 0;   // warp 0, lane 0: the index of the window after the next
   if (wid == 0) {
     fetch_record(0, blockIdx.x);
@@ -461,7 +452,7 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
   }
   copies_done();
   __syncthreads();
-  int slot = 0, buf = 0;
+  int slot = 0, buf = 0, list = 0;
   while (sw.have[slot]) {
     const WinRecord& r = sw.rec[slot];
     const int ns = r.we - r.wb;
@@ -538,7 +529,9 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
         const int o = static_cast<int>(at >> 48), p = static_cast<int>(at >> 20) & 0xffff;
         sw.rest.av[o] = v1;
         sw.rest.bs[o] = bs + 32u * nw - p;
-        sw.rest.end[o] = p + nr;
+        atomicOr(&sw.rest.start[list][p >> 5], 1u << (p & 31));
+        if (p == 0) sw.rest.first[0] = 0;
+        if ((p + nr) >> 5 != static_cast<uint32_t>(p) >> 5) sw.rest.first[(p + nr) >> 5] = static_cast<uint8_t>(o + 1);
       }
       if (c0 + kChunk < na) {
         bs = be = 0;
@@ -556,11 +549,15 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
       }
       __syncthreads();
       const int32_t groups = static_cast<int32_t>(all & 0xfffff), rest = static_cast<int32_t>(all >> 20) & 0xffff;
+      sw.rest.start[list ^ 1][threadIdx.x] = 0u;   // (its last readers are before the barrier above the lists)
+      const uint32_t* start = sw.rest.start[list];
+      list ^= 1;
       // the warps take the steps of both lists in turn: at most one step of each list is short
       const int wsteps = (groups + kGroups - 1) / kGroups, steps = wsteps + (rest + 32 * kGroups - 1) / (32 * kGroups);
+      int from = 0;
       auto load = [&](int q, Step<V>& st) {
-        if (q < wsteps) load_whole(sw.whole, static_cast<int>(all >> 36) & 0xfff, kGroups * q, groups, B.col, bval, st);
-        else load_rest(sw.rest, static_cast<int>(all >> 48), 32 * kGroups * (q - wsteps), rest, B.col, bval, st);
+        if (q < wsteps) load_whole(sw.whole, static_cast<int>(all >> 36) & 0xfff, kGroups * q, groups, B.col, bval, st, from);
+        else load_rest(sw.rest, start, 32 * kGroups * (q - wsteps), rest, B.col, bval, st);
       };
       if (wid < steps) {
         Step<V> cur;
