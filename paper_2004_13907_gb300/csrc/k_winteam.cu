@@ -12,17 +12,17 @@
 //  3. columns and values leave in rank order.
 // The output is sorted by column without a sort, as Algorithm 1's sorted PP (Sec. III-A).
 //
-// Bound by shared memory (the rank lookups and the FP64 atomics: half of the peak wavefronts) and by
-// the barriers between the phases; the atomics alone would take half of the time (1.06 adds of a
-// product per clock per SM, measured). Against one block per row with windows of 4096 entries
-// (k_num_window) and a pass of its own for the columns (k_expand_cols): small windows of any row keep
-// more of them in flight, a list of windows lets the next one's data be fetched ahead, a product stores
-// its column at its rank on the way, so no pass extracts the columns from the bitmap, and whole groups
-// of 32 products of one segment need no search per product. Both kernels -> this one: 30,000^2
-// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 4.58 ms, R-MAT 2^17 (1.09e9) 9.92 -> 6.30 ms, R-MAT 2^19
-// (7.85e9) 77.6 -> 57.5 ms. Of this, finding a product's segment by a bit per segment start instead of a
-// search of the segments' ends (k_num_winteam issued 146 instructions per 32 products): 5.06 -> 4.58,
-// 6.39 -> 6.30, 58.6 -> 57.5.
+// Bound by shared memory (the rank lookups and the sums' compare-and-swaps: 60 % of the peak wavefronts),
+// by the instructions of a product (about 100 per 32 products) and by the FP64 pipe. Against one block per
+// row with windows of 4096 entries (k_num_window) and a pass of its own for the columns (k_expand_cols):
+// small windows of any row keep more of them in flight, a list of windows lets the next one's data be
+// fetched ahead, a product stores its column at its rank on the way, so no pass extracts the columns
+// from the bitmap, whole groups of 32 products of one segment need no search per product, and the
+// others' segment is a popcount of the bits where segments start. Both kernels -> this one: 30,000^2
+// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 4.53 ms, R-MAT 2^17 (1.09e9) 9.92 -> 5.69 ms, R-MAT 2^19
+// (7.85e9) 77.6 -> 54.8 ms. Of this, the bits instead of a search of the segments' ends: 5.06 -> 4.64,
+// 6.39 -> 6.31, 58.6 -> 57.5; the fused sums (add_product_f64) instead of atomicAdd: 4.64 -> 4.53, 6.31 ->
+// 5.69, 57.5 -> 54.8.
 //
 // FP32-compensated plans take the same kernel with FP32 sums and compensations in the eight bytes of a
 // slot (two FP32 atomics a product, separate arrays so that both spread over all banks): R-MAT 2^17
@@ -272,7 +272,9 @@ struct Step {
 };
 
 // Adds the product a * b into the slot of rank r.
-__device__ __forceinline__ void add_product(const Window& win, int r, double a, double b) { atomicAdd(win.vals + r, a * b); }
+__device__ __forceinline__ void add_product(const Window& win, int r, double a, double b) {
+  add_product_f64(win.vals + r, a, b);
+}
 
 // FP32: the error-free product ph + pl, and the sum's own rounding error (TwoSum) rebuilt from the value
 // the atomic returns, as the other compensated kernels do (Dot2 accumulated concurrently).
