@@ -241,6 +241,21 @@ __device__ __forceinline__ int count_clear(uint32_t* bm) {
   return c;
 }
 
+// Bits set in the warp's bitmap (this lane's share).
+template <int PER>
+__device__ __forceinline__ int count_bits(const uint32_t* bm) {
+  using L = Lanes<PER>;
+  int c = 0;
+#pragma unroll
+  for (int q = 0; q < L::NV; ++q) {
+    uint32_t w[L::VW];
+    L::load(bm, q, w);
+#pragma unroll
+    for (int t = 0; t < L::VW; ++t) c += __popc(w[t]);
+  }
+  return c;
+}
+
 // pre[w] = bits set in the bitmap before word w (the per-vector warp scans run side by side);
 // returns the number of bits set.
 template <int PER>
@@ -344,7 +359,9 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   int max_cnt = 0;
   // A row of C over kSmallCap entries sends the whole product to the general path: the warp that finds
   // one says so at once, and the others, which look once per group (a load that the group's work hides),
-  // stop there. Counting on to the end took 1.8 ms of a 30,000^2 product whose every row is too long.
+  // stop there. Counting on to the end took 1.8 ms of a 30,000^2 product whose every row is too long. A row
+  // of many entries of A is looked at after every 32 of them (counting the first row of every warp
+  // to its end: 0.1 ms more).
   bool stop = false;
   auto row_counted = [&](int64_t r, int cnt) {
     if (lane == 0) {
@@ -379,6 +396,11 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
           if (c[u] >= 0 && c[u] < width) atomicOr(&bm0[go[u] * 32 * PER + (c[u] >> 5)], 1u << (c[u] & 31));
           else if (ok[u] && chk) bad = true;   // a column outside its row's column space
       });
+      if (ng == 1 && c0 + 32 < gr.E) {   // a long row: too many entries already?
+        __syncwarp();
+        max_cnt = max(max_cnt, warp_sum(count_bits<PER>(bm0)));
+        if (max_cnt > kSmallCap) return;
+      }
     }
     __syncwarp();
     int cg[4];
