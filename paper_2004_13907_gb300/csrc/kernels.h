@@ -64,6 +64,7 @@ struct SmallGrid {
   int groups;
   bool few;
 };
+constexpr int64_t kSmallMaxCheckBlocks = 1024;   // blocks beyond those that have rows of A
 SmallGrid small_sym_grid(const SmallCsr& A, const SmallCsr& B, int64_t width, int num_sms);
 // Symbolic pass, validation of A and B (when `check`) and the offsets of C's rows, in one kernel:
 // nnz_row[i], loc[i] (row i's offset within its block's run), blk[b] (run b's offset, b <= blocks,

@@ -495,8 +495,9 @@ void plan_bytes_bounds(int64_t m, int64_t a_nnz, int64_t width, int a_rowptr32, 
                                           : 0;
   const int64_t counted = wbits_mb > 0 && width <= kSymWinBits ? (width + kSubCols - 1) / kSubCols : nblocks;
   const int64_t window = ws_rounded(2 * m * counted) + ws_rounded(4 * m) + ws_rounded(4 * a_nnz) + stored;
+  // (the small path's run totals: up to kSmallMaxCheckBlocks of them, whatever m is)
   *lo = fixed;
-  *hi = fixed + tiles + window;
+  *hi = fixed + tiles + window + ws_rounded(8 * (kSmallMaxCheckBlocks + 1));
 }
 
 namespace {

@@ -80,3 +80,23 @@ def test_short_rows_of_a_batch():
         assert np.array_equal(C.row_ptr.cpu().numpy(), ref.row_ptr) and np.array_equal(C.col.cpu().numpy(), ref.col)
         assert np.all(np.abs(C.val.cpu().numpy() - ref.val) <= 1e-12 * ref.mag)
     batch.destroy()
+
+
+@pytest.mark.parametrize("m", [1, 2, 9, 33])
+def test_few_rows_times_a_large_matrix(m):
+    """More blocks than rows of A: the others check B, of which every entry is looked at."""
+    import paper_2004_13907_gb300 as sp
+    n = 5_000
+    A = _lens_matrix([7] * m, n, m)
+    B = _lens_matrix([30] * n, n, m + 1)
+    rp, col, val, *_ = run_gpu(A, B)
+    assert_parity(A, B, rp, col, val)
+    for at in (1, 2_049, 75_001, B.nnz - 1):
+        bad = B.col.copy()
+        bad[at] = n
+        dA = sp.DeviceCSR.from_host(A, "cuda")
+        dB = sp.DeviceCSR.from_host(synth.CSR(n, n, B.row_ptr, bad, B.val), "cuda")
+        with pytest.raises(sp.SpgemmError) as ei:
+            plan = sp.spgemm_plan(dA, dB)
+            sp.spgemm_symbolic(plan)
+        assert ei.value.name == "INVALID_CSR"
