@@ -347,77 +347,78 @@ __global__ void __launch_bounds__(256) k_count(CsrArrays A, CsrArrays B, int run
 
 // Tile histograms are stored class by class: class c's count of tile t at c * ntiles + t.
 //
-// One block: turns the per-tile class counts into per-tile base offsets (in place), writes the class
-// offsets, and scans the per-tile sums. Warp c handles class c, kScanTiles tiles at a time with their
-// loads in flight together (1,024 tiles, cold caches: 29 us with one load at a time, 17 us now).
-constexpr int kScanTiles = 1024;
-template <typename Ld, typename F>
-__device__ __forceinline__ void for_tiles(int64_t ntiles, Ld&& ld, F&& f) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t t0 = 0; t0 < ntiles; t0 += kScanTiles) {
-    decltype(ld(0)) v[kScanTiles / 32];
-#pragma unroll
-    for (int q = 0; q < kScanTiles / 32; ++q) {
-      const int64_t t = t0 + q * 32 + lane;
-      v[q] = t < ntiles ? ld(t) : decltype(ld(0))(0);
-    }
-#pragma unroll
-    for (int q = 0; q < kScanTiles / 32; ++q)
-      if (t0 + q * 32 < ntiles) f(t0 + q * 32 + lane, v[q]);
+// Block c < nclasses turns class c's per-tile counts into offsets within the class (in place) and writes
+// the class's rows to the summary; the block after them scans the per-tile sums. The scatter kernels
+// and the host add the classes before a class up from its rows. Bound by latency: one block for
+// everything, a warp per class, took 18 us for 1,024 tiles, this 4.
+constexpr int kScanThreads = 1024;
+template <typename T, typename Ld, typename St>
+__device__ __forceinline__ T scan_tiles(int64_t ntiles, T* scratch, Ld&& ld, St&& st) {
+  T run = 0;
+  T v = threadIdx.x < ntiles ? ld(threadIdx.x) : T(0);
+  for (int64_t t0 = 0; t0 < ntiles; t0 += kScanThreads) {
+    const int64_t t = t0 + threadIdx.x, after = t + kScanThreads;
+    const T ahead = after < ntiles ? ld(after) : T(0);
+    T total;
+    const T at = run + block_excl_scan<T>(v, scratch, &total);
+    if (t < ntiles) st(t, at);
+    run += total;
+    v = ahead;
+  }
+  return run;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_class_scan(int64_t ntiles, int nclasses, int32_t* tile_hist,
+                                                             const int64_t* tile_sum, const int64_t* tile_max,
+                                                             int64_t* tile_sum_off, Summary* summary) {
+  __shared__ int32_t s_scan[33];
+  __shared__ int64_t s_scan64[33];
+  const int c = blockIdx.x;
+  if (c < nclasses) {
+    int32_t* hist = tile_hist + c * ntiles;
+    const int32_t rows = scan_tiles<int32_t>(ntiles, s_scan, [&](int64_t t) { return hist[t]; },
+                                             [&](int64_t t, int32_t at) { hist[t] = at; });   // rows: below 2^31
+    if (threadIdx.x == 0) summary->class_rows[c] = rows;
+    return;
+  }
+  if (threadIdx.x >= nclasses && threadIdx.x < kMaxClasses) summary->class_rows[threadIdx.x] = 0;
+  const int64_t total = scan_tiles<int64_t>(ntiles, s_scan64, [&](int64_t t) { return tile_sum[t]; },
+                                            [&](int64_t t, int64_t at) {
+                                              if (tile_sum_off) tile_sum_off[t] = at;
+                                            });
+  int64_t mx = 0;
+  if (tile_max) {
+    for (int64_t t = threadIdx.x; t < ntiles; t += kScanThreads) mx = mx > tile_max[t] ? mx : tile_max[t];
+    mx = ~warp_min(~mx);
+    if ((threadIdx.x & 31) == 0) s_scan64[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (threadIdx.x < 32) mx = ~warp_min(~s_scan64[threadIdx.x]);
+  }
+  if (threadIdx.x == 0) {
+    summary->total = total;
+    summary->max_row = mx;
   }
 }
 
-__global__ void __launch_bounds__(544) k_class_scan(int64_t ntiles, int nclasses, int32_t* tile_hist,
-                                                    const int64_t* tile_sum, const int64_t* tile_max,
-                                                    int64_t* tile_sum_off, Summary* summary) {
-  __shared__ int64_t tot[kMaxClasses];
-  __shared__ int64_t off[kMaxClasses + 1];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int32_t* hist = tile_hist + w * ntiles;   // (warp kMaxClasses has no class)
-  auto count = [&](int64_t t) { return hist[t]; };
-  if (w < nclasses) {
-    int64_t s = 0;
-    for_tiles(ntiles, count, [&](int64_t, int32_t v) { s += v; });
-    s = warp_sum(s);
-    if (lane == 0) tot[w] = s;
+// base[c]: where tile t's rows of class c go (all threads of the block call it; ends with a barrier).
+__device__ __forceinline__ void class_bases(const int32_t* tile_hist, int64_t ntiles, int64_t t,
+                                            const Summary* summary, int32_t* base) {
+  if (threadIdx.x < 32) {
+    const int c = threadIdx.x;
+    const int32_t rows = c < kMaxClasses ? static_cast<int32_t>(summary->class_rows[c]) : 0;
+    const int32_t before = warp_incl_scan(rows) - rows;
+    if (c < kMaxClasses) base[c] = before + tile_hist[c * ntiles + t];
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int64_t o = 0;
-    for (int c = 0; c < nclasses; ++c) { off[c] = o; summary->class_off[c] = o; o += tot[c]; }
-    for (int c = nclasses; c <= kMaxClasses; ++c) { off[c] = o; summary->class_off[c] = o; }
-  }
-  __syncthreads();
-  if (w < nclasses) {
-    int32_t run = static_cast<int32_t>(off[w]);   // rows: below 2^31
-    for_tiles(ntiles, count, [&](int64_t t, int32_t v) {
-      const int32_t incl = warp_incl_scan(v);
-      if (t < ntiles) hist[t] = run + incl - v;
-      run += __shfl_sync(0xffffffffu, incl, 31);
-    });
-  } else if (w == kMaxClasses) {
-    int64_t run = 0, mx = 0;
-    if (tile_max) for_tiles(ntiles, [&](int64_t t) { return tile_max[t]; }, [&](int64_t, int64_t v) { mx = mx > v ? mx : v; });
-    for_tiles(ntiles, [&](int64_t t) { return tile_sum[t]; }, [&](int64_t t, int64_t v) {
-      const int64_t incl = warp_incl_scan(v);
-      if (tile_sum_off && t < ntiles) tile_sum_off[t] = run + incl - v;
-      run += __shfl_sync(0xffffffffu, incl, 31);
-    });
-    mx = ~warp_min(~mx);
-    if (lane == 0) {
-      summary->total = run;
-      summary->max_row = mx;
-    }
-  }
 }
 
 __global__ void __launch_bounds__(256) k_scatter_sym(DevCsr A, ClassParams cp, const int64_t* P,
-                                                     const int32_t* tile_hist, int32_t* perm) {
+                                                     const int32_t* tile_hist, const Summary* summary,
+                                                     int32_t* perm) {
   __shared__ int32_t base[kMaxClasses];
   __shared__ int32_t s_cnt[8][kMaxClasses];
   const int64_t t = blockIdx.x;
-  if (threadIdx.x < kMaxClasses) base[threadIdx.x] = tile_hist[threadIdx.x * int64_t(gridDim.x) + t];
-  __syncthreads();
+  class_bases(tile_hist, gridDim.x, t, summary, base);
   for (int r = 0; r < kTileRows / 256; ++r) {
     const int64_t row = t * kTileRows + r * 256 + threadIdx.x;
     const bool valid = row < A.rows;
@@ -490,14 +491,13 @@ __global__ void __launch_bounds__(256) k_num_tiles(DevCsr A, ClassParams cp, con
 // Row offsets of C (exclusive scan of nnz(C_i), int64) and the numeric class scatter.
 __global__ void __launch_bounds__(256) k_scatter_num(DevCsr A, ClassParams cp, const int64_t* P,
                                                      const int32_t* nnz_row, const int32_t* tile_hist,
-                                                     const int64_t* tile_sum_off, int32_t* perm,
-                                                     int64_t* c_off) {
+                                                     const int64_t* tile_sum_off, const Summary* summary,
+                                                     int32_t* perm, int64_t* c_off) {
   __shared__ int32_t base[kMaxClasses];
   __shared__ int32_t s_cnt[8][kMaxClasses];
   __shared__ int64_t scratch[33];
   const int64_t t = blockIdx.x;
-  if (threadIdx.x < kMaxClasses) base[threadIdx.x] = tile_hist[threadIdx.x * int64_t(gridDim.x) + t];
-  __syncthreads();
+  class_bases(tile_hist, gridDim.x, t, summary, base);
   int64_t carry = tile_sum_off[t];
   for (int r = 0; r < kTileRows / 256; ++r) {
     const int64_t row = t * kTileRows + r * 256 + threadIdx.x;
@@ -608,16 +608,16 @@ int launch_count(const CsrArrays& A, const CsrArrays& B, int check, int64_t* a64
 int launch_class_scan(int64_t ntiles, int nclasses, int32_t* tile_hist, const int64_t* tile_sum,
                        const int64_t* tile_max, int64_t* tile_sum_off, Summary* summary,
                        cudaStream_t s) {
-  k_class_scan<<<1, 544, 0, s>>>(ntiles, nclasses, tile_hist, tile_sum, tile_max, tile_sum_off,
+  k_class_scan<<<nclasses + 1, kScanThreads, 0, s>>>(ntiles, nclasses, tile_hist, tile_sum, tile_max, tile_sum_off,
                                  summary);
   return 1;
 }
 
 int launch_scatter_sym(const DevCsr& A, ClassParams cp, const int64_t* P, const int32_t* tile_hist,
-                        int32_t* perm, cudaStream_t s) {
+                        const Summary* summary, int32_t* perm, cudaStream_t s) {
   const int64_t ntiles = (A.rows + kTileRows - 1) / kTileRows;
   if (ntiles == 0) return 0;
-  k_scatter_sym<<<static_cast<unsigned>(ntiles), 256, 0, s>>>(A, cp, P, tile_hist, perm);
+  k_scatter_sym<<<static_cast<unsigned>(ntiles), 256, 0, s>>>(A, cp, P, tile_hist, summary, perm);
   return 1;
 }
 
@@ -631,12 +631,12 @@ int launch_num_tiles(const DevCsr& A, ClassParams cp, const int64_t* P, const in
 }
 
 int launch_scatter_num(const DevCsr& A, ClassParams cp, const int64_t* P, const int32_t* nnz_row,
-                        const int32_t* tile_hist, const int64_t* tile_sum_off, int32_t* perm,
-                        int64_t* c_off, cudaStream_t s) {
+                        const int32_t* tile_hist, const int64_t* tile_sum_off, const Summary* summary,
+                        int32_t* perm, int64_t* c_off, cudaStream_t s) {
   const int64_t ntiles = (A.rows + kTileRows - 1) / kTileRows;
   if (ntiles == 0) return 0;
   k_scatter_num<<<static_cast<unsigned>(ntiles), 256, 0, s>>>(A, cp, P, nnz_row, tile_hist,
-                                                              tile_sum_off, perm, c_off);
+                                                              tile_sum_off, summary, perm, c_off);
   return 1;
 }
 

@@ -28,7 +28,7 @@ struct CsrArrays {
 
 // Summary the host reads back after the plan and after the symbolic pass.
 struct Summary {
-  int64_t class_off[kMaxClasses + 1];
+  int64_t class_rows[kMaxClasses];
   int64_t total;          // sum of P_i (plan) or of nnz(C_i) (symbolic)
   int64_t max_row;        // max P_i
   unsigned long long cls_sums[kMaxClasses][3];  // per numeric class: sum P_i, sum nnz(A_i), sum nnz(C_i)
@@ -104,13 +104,13 @@ int launch_class_scan(int64_t ntiles, int nclasses, int32_t* tile_hist, const in
                        const int64_t* tile_max, int64_t* tile_sum_off, Summary* summary,
                        cudaStream_t s);
 int launch_scatter_sym(const DevCsr& A, ClassParams cp, const int64_t* P, const int32_t* tile_hist,
-                        int32_t* perm, cudaStream_t s);
+                        const Summary* summary, int32_t* perm, cudaStream_t s);
 int launch_num_tiles(const DevCsr& A, ClassParams cp, const int64_t* P, const int32_t* nnz_row,
                       int32_t* tile_hist, int64_t* tile_sum, unsigned long long* cls_sums,
                       cudaStream_t s);
 int launch_scatter_num(const DevCsr& A, ClassParams cp, const int64_t* P, const int32_t* nnz_row,
-                        const int32_t* tile_hist, const int64_t* tile_sum_off, int32_t* perm,
-                        int64_t* c_off, cudaStream_t s);
+                        const int32_t* tile_hist, const int64_t* tile_sum_off, const Summary* summary,
+                        int32_t* perm, int64_t* c_off, cudaStream_t s);
 int launch_write_rowptr(const int64_t* c_off, int64_t m1, void* out, int idx64, cudaStream_t s);
 
 // ---- symbolic kernels (k_symbolic.cu). Each handles perm[start, start+count).

@@ -40,6 +40,12 @@ spgemm_status error_bits_status(uint32_t err) {
   return SPGEMM_OK;
 }
 
+// Where each class's rows start in the permutation, and their number last.
+void class_offsets(const Summary& h, int64_t (&off)[kMaxClasses + 1]) {
+  off[0] = 0;
+  for (int c = 0; c < kMaxClasses; ++c) off[c + 1] = off[c] + h.class_rows[c];
+}
+
 int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 }  // namespace
@@ -332,12 +338,12 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
                           &p->summary->err, s);
     nl += launch_class_scan(p->ntiles, kSymNumClasses, p->tile_hist, p->tile_sum, p->tile_max, nullptr,
                             p->summary, s);
-    nl += launch_scatter_sym(p->A, p->cp, p->P, p->tile_hist, p->perm_s, s);
+    nl += launch_scatter_sym(p->A, p->cp, p->P, p->tile_hist, p->summary, p->perm_s, s);
     stage_end(p, SPGEMM_STAGE_COUNT, nl, s);
     if ((st = cuda_status(cudaGetLastError(), "launching the plan kernels")) != SPGEMM_OK) return st;
     if ((st = read_summary(p, &h, s)) != SPGEMM_OK) return st;
     if (h.err) return error_bits_status(h.err);
-    std::memcpy(p->sym_off, h.class_off, sizeof(p->sym_off));
+    class_offsets(h, p->sym_off);
     p->total_products = h.total;
     p->max_row_products = h.max_row;
   } else if (o.validate) {
@@ -461,14 +467,14 @@ spgemm_status symbolic_run(spgemm_plan_s* p, cudaStream_t s) {
     nl = launch_num_tiles(p->A, p->cp, p->P, p->nnz_row, p->tile_hist, p->tile_sum, &p->summary->cls_sums[0][0], s);
     nl += launch_class_scan(p->ntiles, kNumNumClasses, p->tile_hist, p->tile_sum, nullptr, p->tile_sum_off,
                             p->summary, s);
-    nl += launch_scatter_num(p->A, p->cp, p->P, p->nnz_row, p->tile_hist, p->tile_sum_off, p->perm_n,
-                             p->c_off, s);
+    nl += launch_scatter_num(p->A, p->cp, p->P, p->nnz_row, p->tile_hist, p->tile_sum_off, p->summary,
+                             p->perm_n, p->c_off, s);
     stage_end(p, SPGEMM_STAGE_SYM_SCAN, nl, s);
     if ((st = cuda_status(cudaGetLastError(), "launching the symbolic kernels")) != SPGEMM_OK) return st;
     Summary h;
     if ((st = read_summary(p, &h, s)) != SPGEMM_OK) return st;
     if (h.err) return error_bits_status(h.err);
-    std::memcpy(p->num_off, h.class_off, sizeof(p->num_off));
+    class_offsets(h, p->num_off);
     std::memcpy(p->cls_sums, h.cls_sums, sizeof(p->cls_sums));
     p->nnz_c = h.total;
   } else {
