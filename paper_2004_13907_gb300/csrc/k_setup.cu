@@ -161,35 +161,43 @@ __device__ __forceinline__ int32_t aggregated_slot(int32_t* counters, int cls, b
   return base + rank;
 }
 
-// Places of 256 consecutive rows (one per thread) within their classes, in row order, from base[class],
-// which moves past them: neighbouring rows of a class stay neighbours in the permutation (the merge
-// kernel writes a warp's rows as one run). cnt: a counter per warp and class. Contains __syncthreads.
-__device__ __forceinline__ int32_t ordered_slot(int32_t* base, int32_t (*cnt)[kMaxClasses], int cls, bool valid) {
+// Rows of a tile per thread of the kernels of 256 threads below: row r * 256 + threadIdx.x. The loads of all
+// of them are under way before the first is ranked, and the tile's rows are ranked at once (2^20 rows,
+// with a ranking of its own, and three barriers, for every 256 rows: k_scatter_num 19 us, now 16,
+// k_scatter_sym 11, now 9).
+constexpr int kRowsPer = kTileRows / 256;
+constexpr int kGroups = kTileRows / 32;   // of 32 consecutive rows
+static_assert(kGroups == 32, "a lane per group");
+
+// Places of a tile's rows within their classes, in row order, from base[class]: neighbouring rows of a class
+// stay neighbours in the permutation (the merge kernel writes a warp's rows as one run). cls < 0: no row.
+// cnt: a counter per group and class. Contains __syncthreads.
+__device__ __forceinline__ void ordered_slots(const int32_t* base, int32_t (*cnt)[kMaxClasses],
+                                              const int (&cls)[kRowsPer], int32_t (&pos)[kRowsPer]) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane < kMaxClasses) cnt[wid][lane] = 0;
-  __syncwarp();
-  unsigned peers = 0;
-  for (unsigned todo = __ballot_sync(0xffffffffu, valid); todo;) {
-    const int lc = __shfl_sync(0xffffffffu, cls, __ffs(todo) - 1);
-    const unsigned same = __ballot_sync(0xffffffffu, valid && cls == lc);
-    if (valid && cls == lc) peers = same;
-    if (lane == 0) cnt[wid][lc] = __popc(same);
-    todo &= ~same;
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r) {
+    int32_t* mine = cnt[r * 8 + wid];
+    if (lane < kMaxClasses) mine[lane] = 0;
+    __syncwarp();
+    pos[r] = 0;
+    for (unsigned todo = __ballot_sync(0xffffffffu, cls[r] >= 0); todo;) {
+      const int lc = __shfl_sync(0xffffffffu, cls[r], __ffs(todo) - 1);
+      const unsigned same = __ballot_sync(0xffffffffu, cls[r] == lc);
+      if (cls[r] == lc) pos[r] = __popc(same & ((1u << lane) - 1u));
+      if (lane == 0) mine[lc] = __popc(same);
+      todo &= ~same;
+    }
   }
   __syncthreads();
-  int32_t at = 0;
-  if (valid) {
-    at = base[cls] + __popc(peers & ((1u << lane) - 1u));
-    for (int w = 0; w < wid; ++w) at += cnt[w][cls];
+  for (int c = wid; c < kMaxClasses; c += 8) {
+    const int32_t v = cnt[lane][c];
+    cnt[lane][c] = base[c] + warp_incl_scan(v) - v;
   }
   __syncthreads();
-  if (threadIdx.x < kMaxClasses) {
-    int32_t all = 0;
-    for (int w = 0; w < 8; ++w) all += cnt[w][threadIdx.x];
-    base[threadIdx.x] += all;
-  }
-  __syncthreads();
-  return at;
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r)
+    if (cls[r] >= 0) pos[r] += cnt[r * 8 + wid][cls[r]];
 }
 
 // Rows with more entries than this are counted by the whole block of k_count.
@@ -416,21 +424,25 @@ __global__ void __launch_bounds__(256) k_scatter_sym(DevCsr A, ClassParams cp, c
                                                      const int32_t* tile_hist, const Summary* summary,
                                                      int32_t* perm) {
   __shared__ int32_t base[kMaxClasses];
-  __shared__ int32_t s_cnt[8][kMaxClasses];
+  __shared__ int32_t s_cnt[kGroups][kMaxClasses];
   const int64_t t = blockIdx.x;
-  class_bases(tile_hist, gridDim.x, t, summary, base);
-  for (int r = 0; r < kTileRows / 256; ++r) {
+  int cls[kRowsPer];
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r) {
     const int64_t row = t * kTileRows + r * 256 + threadIdx.x;
-    const bool valid = row < A.rows;
-    int cls = 0;
-    if (valid) {
+    cls[r] = -1;
+    if (row < A.rows) {
       int64_t a0, na;
       clamped_row(A, row, a0, na);   // the same row length k_count classified (before validation's verdict)
-      cls = sym_class(P[row], na > 0x7fffffff ? 0x7fffffff : static_cast<int32_t>(na), row_params(cp, row));
+      cls[r] = sym_class(P[row], na > 0x7fffffff ? 0x7fffffff : static_cast<int32_t>(na), row_params(cp, row));
     }
-    const int32_t pos = ordered_slot(base, s_cnt, cls, valid);
-    if (valid) perm[pos] = static_cast<int32_t>(row);
   }
+  class_bases(tile_hist, gridDim.x, t, summary, base);
+  int32_t pos[kRowsPer];
+  ordered_slots(base, s_cnt, cls, pos);
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r)
+    if (cls[r] >= 0) perm[pos[r]] = static_cast<int32_t>(t * kTileRows + r * 256 + threadIdx.x);
 }
 
 __global__ void __launch_bounds__(256) k_num_tiles(DevCsr A, ClassParams cp, const int64_t* P,
@@ -494,32 +506,46 @@ __global__ void __launch_bounds__(256) k_scatter_num(DevCsr A, ClassParams cp, c
                                                      const int64_t* tile_sum_off, const Summary* summary,
                                                      int32_t* perm, int64_t* c_off) {
   __shared__ int32_t base[kMaxClasses];
-  __shared__ int32_t s_cnt[8][kMaxClasses];
-  __shared__ int64_t scratch[33];
+  __shared__ int32_t s_cnt[kGroups][kMaxClasses];
+  __shared__ int64_t s_z[kGroups];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t t = blockIdx.x;
-  class_bases(tile_hist, gridDim.x, t, summary, base);
-  int64_t carry = tile_sum_off[t];
-  for (int r = 0; r < kTileRows / 256; ++r) {
+  int cls[kRowsPer];
+  int32_t z[kRowsPer];
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r) {
     const int64_t row = t * kTileRows + r * 256 + threadIdx.x;
-    const bool valid = row < A.rows;
-    int cls = 0;
-    int64_t z = 0;
-    if (valid) {
+    cls[r] = -1;
+    z[r] = 0;
+    if (row < A.rows) {
       const int64_t na = A.rp[row + 1] - A.rp[row];
-      z = nnz_row[row];
-      cls = num_class(P[row], na > 0x7fffffff ? 0x7fffffff : static_cast<int32_t>(na),
-                      static_cast<int32_t>(z), cp);
+      z[r] = nnz_row[row];
+      cls[r] = num_class(P[row], na > 0x7fffffff ? 0x7fffffff : static_cast<int32_t>(na), z[r], cp);
     }
-    int64_t tot;
-    const int64_t ex = block_excl_scan<int64_t>(z, scratch, &tot);
-    if (valid) {
-      c_off[row] = carry + ex;
-      if (row == A.rows - 1) c_off[A.rows] = carry + ex + z;
-    }
-    carry += tot;
-    const int32_t pos = ordered_slot(base, s_cnt, cls, valid);
-    if (valid) perm[pos] = static_cast<int32_t>(row);
   }
+  const int64_t carry = tile_sum_off[t];
+  int64_t incl[kRowsPer];
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r) {
+    incl[r] = warp_incl_scan(static_cast<int64_t>(z[r]));
+    if (lane == 31) s_z[r * 8 + wid] = incl[r];
+  }
+  class_bases(tile_hist, gridDim.x, t, summary, base);   // (ends with a barrier)
+  const int64_t group = s_z[lane], before = warp_incl_scan(group) - group;
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r) {
+    const int64_t row = t * kTileRows + r * 256 + threadIdx.x;
+    const int64_t end = carry + __shfl_sync(0xffffffffu, before, r * 8 + wid) + incl[r];
+    if (row < A.rows) {
+      c_off[row] = end - z[r];
+      if (row == A.rows - 1) c_off[A.rows] = end;
+    }
+  }
+  int32_t pos[kRowsPer];
+  ordered_slots(base, s_cnt, cls, pos);
+#pragma unroll
+  for (int r = 0; r < kRowsPer; ++r)
+    if (cls[r] >= 0) perm[pos[r]] = static_cast<int32_t>(t * kTileRows + r * 256 + threadIdx.x);
 }
 
 __global__ void __launch_bounds__(256) k_collect_flagged(const int32_t* __restrict__ perm, int64_t count,
