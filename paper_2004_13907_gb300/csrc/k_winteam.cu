@@ -19,14 +19,14 @@
 // fetched ahead, a product stores its column at its rank on the way, so no pass extracts the columns
 // from the bitmap, whole groups of 32 products of one segment need no search per product, and the
 // others' segment is a popcount of the bits where segments start. Both kernels -> this one: 30,000^2
-// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 4.53 ms, R-MAT 2^17 (1.09e9) 9.92 -> 5.69 ms, R-MAT 2^19
-// (7.85e9) 77.6 -> 54.8 ms. Of this, the bits instead of a search of the segments' ends: 5.06 -> 4.64,
+// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 4.21 ms, R-MAT 2^17 (1.09e9) 9.92 -> 5.68 ms, R-MAT 2^19
+// (7.85e9) 77.6 -> 51.8 ms. Of this, the bits instead of a search of the segments' ends: 5.06 -> 4.64,
 // 6.39 -> 6.31, 58.6 -> 57.5; the fused sums (add_product_f64) instead of atomicAdd: 4.64 -> 4.53, 6.31 ->
 // 5.69, 57.5 -> 54.8.
 //
 // FP32-compensated plans take the same kernel with FP32 sums and compensations in the eight bytes of a
 // slot (two FP32 atomics a product, separate arrays so that both spread over all banks): R-MAT 2^17
-// 7.93 -> 5.73 ms. A slot that also needs the sum of |p| and the term count takes sixteen bytes and its
+// 7.93 -> 5.45 ms. A slot that also needs the sum of |p| and the term count takes sixteen bytes and its
 // windows half the entries; with mixed signs (R-MAT 2^17 of 8 edges a vertex) 4.51 -> 3.50 ms.
 #include <type_traits>
 
@@ -38,20 +38,22 @@ namespace spg {
 namespace {
 
 // A window's size against the number of windows an SM works on at once (one per block; a block is idle
-// while its window's ranks are made, at its barriers and while it writes out). Measured with a search of
-// the segments' ends, ms of the numeric pass on the 30,000^2 uniform product (d = 5e-3), R-MAT 2^17 and R-MAT 2^19:
-//   4 warps, 2048 entries, 32 sub-blocks, 6 blocks per SM: 5.06, 6.39, 58.5 (taken)
-//   4 warps, 1536 entries, 7 blocks: 5.63, 6.62, 62.1;  1152 entries, 8 blocks: 5.82, 6.99, 66.7
-//   4 warps, 1920 entries, 64 sub-blocks, 5 blocks: 5.70, 6.85, 61.5
-//   2 warps, 1024 entries, 16 sub-blocks, 12 blocks: 6.93, 6.69, 69.0
-//   8 warps, 2688 entries, 64 sub-blocks, 4 blocks: 4.84, 6.89, 58.8
-constexpr int kWinCap = 2048;      // entries of C per window (>= kSubCols)
-constexpr int kWinSpan = 32;       // sub-blocks per window
-constexpr int kTeam = 4;           // warps per block: one window at a time
-constexpr int kTeamBlocks = 6;     // blocks per SM
+// while its window's ranks are made, at its barriers and while it writes out), and the products a warp
+// has under way. Measured, ms of the numeric pass on the 30,000^2 uniform product (d = 5e-3), R-MAT 2^17,
+// the same FP32-compensated, and R-MAT 2^19:
+//   8 warps, 4096 entries, 64 sub-blocks, 3 blocks per SM, 3 groups a step: 4.21, 5.68, 5.45, 51.8 (taken)
+//   the same with 2 groups: 4.17, 5.74, 5.68, 51.7;  3584 entries: 4.17, 5.93, 5.68, 53.3
+//   8 warps, 4096 entries, 32 sub-blocks, 3 blocks: 3.97, 5.87, 5.90, 54.5;  3072, 4 blocks: 4.06, 5.83, 5.53, 55.8
+//   8 warps, 2560 entries, 64 sub-blocks, 4 blocks: 4.45, 6.09, 5.69, 54.4
+//   4 warps, 2048 entries, 32 sub-blocks, 6 blocks: 4.53, 5.69, 5.75, 54.8;  3 groups: 4.69, 5.66, 5.60, 55.2
+//   16 warps, 4096 entries, 64 sub-blocks, 2 blocks: 4.78, 7.34, 6.35, 64.5
+constexpr int kWinCap = 4096;      // entries of C per window (>= kSubCols)
+constexpr int kWinSpan = 64;       // sub-blocks per window
+constexpr int kTeam = 8;           // warps per block: one window at a time
+constexpr int kTeamBlocks = 3;     // blocks per SM
 constexpr int kChunk = kTeam * 32; // A entries per chunk, one per thread
 constexpr int kRankStep = kWinSpan / 4 / kTeam;   // runs of four sub-blocks per warp
-constexpr int kGroups = 2;         // groups of 32 products per step; a warp has two steps under way
+constexpr int kGroups = 3;         // groups of 32 products per step; a warp has two steps under way
 constexpr int kSlots = 3;          // window records in shared memory: this one, the next, the one after
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWideCap = kWinCap / 2;   // entries of C per window of wide slots
@@ -86,7 +88,7 @@ struct RestList {
   V av[kChunk];
   uint32_t bs[kChunk];         // start in B less the number of the segment's first product
   uint32_t start[2][kChunk];   // bit per product: a segment starts there (this chunk's, and zeros for the next)
-  uint8_t first[kChunk];       // per 32 products: the first segment that starts among them. None has 32
+  uint16_t first[kChunk];      // per 32 products: the first segment that starts among them. None has 32
 };                             // products, so one does
 
 template <typename V>
@@ -533,7 +535,7 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
         sw.rest.bs[o] = bs + 32u * nw - p;
         atomicOr(&sw.rest.start[list][p >> 5], 1u << (p & 31));
         if (p == 0) sw.rest.first[0] = 0;
-        if ((p + nr) >> 5 != static_cast<uint32_t>(p) >> 5) sw.rest.first[(p + nr) >> 5] = static_cast<uint8_t>(o + 1);
+        if ((p + nr) >> 5 != static_cast<uint32_t>(p) >> 5) sw.rest.first[(p + nr) >> 5] = static_cast<uint16_t>(o + 1);
       }
       if (c0 + kChunk < na) {
         bs = be = 0;

@@ -1,5 +1,5 @@
 """FP32-compensated rows over the list of windows: slots of a sum and a compensation where every product
-is non-negative and few (windows of 2,048 entries), wide slots (1,024 entries) where the signs mix or a
+is non-negative and few (windows of 4,096 entries), wide slots (2,048 entries) where the signs mix or a
 row of A has more entries than the count bound allows (about 4,000); and values whose signs change
 between numeric passes of one plan."""
 
@@ -36,11 +36,11 @@ def _within(A, B, rp, col, val):
 
 @pytest.mark.parametrize("signed", [False, True])
 @pytest.mark.parametrize("n", [1_023, 1_025, 32_769, 90_000])
-@pytest.mark.parametrize("fill", [1, 1_024, 4_096])
+@pytest.mark.parametrize("fill", [1, 2_048, 4_096])
 def test_slots(n, signed, fill):
     import paper_2004_13907_gb300 as sp
     k = 6_000
-    A = _matrix(8, k, [1, 127, 128, 129, 300, 3_900, 4_200, 6_000], n, signed)
+    A = _matrix(8, k, [1, 255, 256, 257, 300, 3_900, 4_200, 6_000], n, signed)
     B = _matrix(k, n, np.random.default_rng(n + 1).integers(0, 60, k), n + 2, signed)
     rp, col, val, _, info, _ = run_gpu(A, B, sp.spgemm_opts_default(force_window=1, window_hash_fill=fill), prec="f32c")
     assert sum(info["num_class_rows"][:4]) == A.rows

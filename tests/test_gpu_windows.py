@@ -1,7 +1,7 @@
 """The numeric pass over a list of windows (FP64 rows whose bitmaps are all stored) against the
-oracle: column spaces around a sub-block (1,024 columns) and a window (32 of them), up to 2^20 columns;
+oracle: column spaces around a sub-block (1,024 columns) and a window (64 of them), up to 2^20 columns;
 segments of B from single products to many whole groups of 32; rows of one and of several chunks of A
-entries (128); window sizes, no split table; and the same product without stored bitmaps, which takes
+entries (256); window sizes, no split table; and the same product without stored bitmaps, which takes
 the other windowed kernel."""
 
 import numpy as np
@@ -37,8 +37,8 @@ def _skewed(k, n, seed):
     return synth.CSR(k, n, rp, col, rng.random(col.size) * 2 - 1)
 
 
-@pytest.mark.parametrize("n", [1, 31, 1_000, 1_024, 1_025, 32_768, 32_769, 65_536, 70_001, 262_144, 1 << 20])
-@pytest.mark.parametrize("na", [5, 128, 129, 300])
+@pytest.mark.parametrize("n", [1, 31, 1_000, 1_024, 1_025, 32_769, 65_536, 65_537, 70_001, 262_144, 1 << 20])
+@pytest.mark.parametrize("na", [5, 128, 256, 257, 300])
 def test_window_list(n, na):
     k = 400
     A = synth.uniform_random(30, k, na / k, seed=n + na)
