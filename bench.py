@@ -68,8 +68,8 @@ def _peaks():
 
 
 def _fp64_pipe(products: int, ms: float, sm_count: int, sm_mhz) -> dict:
-    """The windowed numeric pass against GB300's FP64 pipe: every partial product costs two FP64
-    operations there (the product a_ik * b_kj and the add inside the shared atomic), and the pipe
+    """The windowed numeric pass against GB300's FP64 pipe: every partial product is two FP64
+    operations (the product a_ik * b_kj and its add; one fused instruction where they meet), and the pipe
     executes 2 lanes per clock per SM (1.25 TFLOP/s counted as FMA), at the sampled SM clock."""
     mhz = float(sm_mhz) if sm_mhz else 2070.0
     peak = 2.0 * sm_count * mhz * 1e6
@@ -126,14 +126,19 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(rows)}
 
 
-def _traffic(alg_bytes: int, root: str = ROOT):
-    """DRAM bytes of the windowed pass (k_num_window + k_expand_cols) per launch: the committed
-    small-case record (R-MAT 2^17, one-pass ncu launch list) gives DRAM bytes per algorithmic byte,
-    scaled to this launch by its algorithmic bytes; None when the record was taken on another
-    version of the kernel source."""
+# The windowed numeric pass: one kernel over a list of windows, or, for plans whose windowed rows do not all
+# have a stored bitmap, one block per row and a second kernel for the columns.
+WINDOW_PASS = {False: ("k_num_winteam", "k_num_winteam_rmat17.md", "k_winteam.cu"),
+               True: ("k_num_window + k_expand_cols", "k_num_window_rmat17.md", "k_window.cu")}
+
+
+def _traffic(alg_bytes: int, root: str = ROOT, profile: str = "k_num_window_rmat17.md", source: str = "k_window.cu"):
+    """DRAM bytes of the windowed pass per launch: the committed small-case record (R-MAT 2^17, one-pass
+    ncu launch list) gives DRAM bytes per algorithmic byte, scaled to this launch by its algorithmic
+    bytes; None when the record was taken on another version of the kernel source."""
     import hashlib
-    path = os.path.join(root, "profiles", "k_num_window_rmat17.md")
-    src = os.path.join(root, "paper_2004_13907_gb300", "csrc", "k_window.cu")
+    path = os.path.join(root, "profiles", profile)
+    src = os.path.join(root, "paper_2004_13907_gb300", "csrc", source)
     try:
         want = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
         fields = {}
@@ -173,8 +178,7 @@ def _dist():
 
 
 def _window_bytes(info: dict, vbytes: int = 8) -> tuple:
-    """Algorithmic bytes of the windowed numeric pass (k_num_window, and k_expand_cols for the
-    columns of rows whose bitmap the symbolic pass stored): per row 8 (its A row pointers), per
+    """Algorithmic bytes of the windowed numeric pass: per row 8 (its A row pointers), per
     A entry 4 + v (column, value) + 8 (start and end of the named B row), per partial product
     4 + v (the gathered B column and value), per entry of C 4 + v (column, value); v = 8 (FP64)
     or 4 (FP32)."""
@@ -239,6 +243,7 @@ def _product_config(wl: str, args, sp, torch, steps: int, warmup: int, cpu_err: 
             out.append((name, plan, C))
         return out
 
+    expanded = {}   # per product: the columns were written by a pass of their own
     for _ in range(warmup):
         for name, plan, C in step(opts):
             sp.spgemm_plan_destroy(plan)
@@ -265,7 +270,9 @@ def _product_config(wl: str, args, sp, torch, steps: int, warmup: int, cpu_err: 
                     launches += info["kernel_launches"]
                 else:
                     step_st = {}
-                    for k, (ms, _) in sp.spgemm_plan_get_timings(plan).items():
+                    for k, (ms, n_launched) in sp.spgemm_plan_get_timings(plan).items():
+                        if k == "num_expand":
+                            expanded[name] = n_launched > 0
                         key = (name, "num_window" if k == "num_expand" else k)   # the expansion completes the pass
                         step_st[key] = step_st.get(key, 0.0) + ms
                     for key, ms in step_st.items():
@@ -288,7 +295,7 @@ def _product_config(wl: str, args, sp, torch, steps: int, warmup: int, cpu_err: 
            "stage_timing": "stage events in as many further steps (the timed steps run default options)"}
     if dom_stage == "num_window":
         wb, _ = _window_bytes(infos[dom_name], _vbytes(precs[dom_name]))
-        out["roofline"] = {"bound": "hbm", "kernel": f"k_num_window + k_expand_cols ({dom_name})",
+        out["roofline"] = {"bound": "hbm", "kernel": f"{WINDOW_PASS[expanded.get(dom_name, False)][0]} ({dom_name})",
                            "achieved": round(wb / (dom_ms * 1e-3) / 1e9, 1), "peak": peak, "unit": "GB/s",
                            "frac": round(wb / (dom_ms * 1e-3) / 1e9 / peak, 4), "algorithmic_bytes": wb,
                            "launch_ms": round(dom_ms, 4)}
@@ -497,6 +504,7 @@ def run_ours(args):
             tim = sp.spgemm_plan_get_timings(plan)
             launches += info["kernel_launches"]
             d = per.setdefault(name, {"info": info, "stages": {}, "rows": M.rows})
+            d["expanded"] = tim["num_expand"][1] > 0
             for k, (ms, nl) in tim.items():
                 d["stages"].setdefault(k, []).append(ms)
             sp.spgemm_plan_destroy(plan)
@@ -526,14 +534,15 @@ def run_ours(args):
     if dom_stage == "num_window":
         bytes_, wprods = _window_bytes(per[dom_mat]["info"], _vbytes(precs[dom_mat]))
         achieved = bytes_ / (dom_ms * 1e-3) / 1e9
-        roof = {"bound": "hbm", "kernel": f"k_num_window + k_expand_cols ({dom_mat})",
+        kernel, profile, source = WINDOW_PASS[per[dom_mat]["expanded"]]
+        roof = {"bound": "hbm", "kernel": f"{kernel} ({dom_mat})",
                 "achieved": round(achieved, 1),
                 "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
                 "peak_source": f"{peak_kind} hbm_gbs", "algorithmic_bytes": bytes_,
                 "launch_ms": round(dom_ms, 4), "traffic": None, "traffic_source": None}
         if all(p == "f64" for p in precs.values()):
-            roof["traffic"] = _traffic(bytes_)
-            roof["traffic_source"] = ("R-MAT 2^17 DRAM bytes per algorithmic byte (profiles/k_num_window_rmat17.md) x "
+            roof["traffic"] = _traffic(bytes_, profile=profile, source=source)
+            roof["traffic_source"] = (f"R-MAT 2^17 DRAM bytes per algorithmic byte (profiles/{profile}) x "
                                       "this launch's algorithmic bytes; B fits L2 at 2^17, so a lower bound here")
         if all(p == "f64" for p in precs.values()):
             roof.update(_fp64_pipe(wprods, dom_ms,

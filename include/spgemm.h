@@ -101,7 +101,7 @@ typedef struct spgemm_opts {
                                  shared table (default 32; 0 disables the class) */
   int32_t warp_max;           /* symbolic: rows with min(P_i, n) <= this use a warp table;
                                  numeric: rows with nnz(C_i) <= warp_max/2 (default 1024) */
-  int32_t block_max;          /* rows up to this size use a block-wide hash table; larger
+  int32_t block_max;          /* rows up to this size use a block-wide table; larger
                                  rows take the windowed path (default 2048, at most 4096) */
   int32_t window_hash_fill;   /* windowed rows: consecutive column blocks are merged into one
                                  window while it holds at most this many entries of C (default
@@ -332,7 +332,7 @@ spgemm_status spgemm_autotune_batch(int64_t n_jobs, const spgemm_csr_in* A, cons
 
 /* ---- Format front-ends. The paper's CPU side reorganises the input matrices into its streamed
  * row bundles and back (Sec. II); here the reorganisation between formats runs on the device, as
- * a stable radix sort of the entries by their new row (see formats.cu). CSC is the CSR of the
+ * a stable radix sort of the entries by their new place (see formats.cu). CSC is the CSR of the
  * transpose, so a product of CSC matrices needs no conversion: C = A*B in CSC is
  * C^T = B^T * A^T in CSR, i.e. spgemm_plan(B_csc viewed as CSR, A_csc viewed as CSR).
  *

@@ -7,11 +7,12 @@
 //  * tiny  : P_i <= 32: one warp, one product per lane; equal columns are grouped with a
 //            warp match and summed by the lowest lane of the group in product order; the
 //            output position is the number of smaller columns in the row.
+//  * micro, merge : one thread per row of at most 8 entries of A, a merge of the B rows.
 //  * warp  : one warp per row, a shared hash table (column -> FP64 sum) of 64/256/1024
 //            slots, then the occupied slots are compacted and bitonic-sorted by column.
 //  * block : one block per row: bitmaps of the row's columns and a rank-indexed array (rows of at
 //            most 2^22 columns), or a hash table of 2048 or 8192 slots, compaction, bitonic sort.
-//  * window: rows with more entries than a block table (k_window.cu).
+//  * window: rows with more entries than a block table (k_winteam.cu, k_window.cu).
 // Sums are accumulated with shared-memory FP64 atomics, so their order (and the last bits of
 // a value) can change from run to run; the pattern is always exact.
 #include "enumerate.cuh"

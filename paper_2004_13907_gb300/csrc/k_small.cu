@@ -17,7 +17,8 @@
 // Each block of the symbolic kernel takes a contiguous run of rows and ends with their offsets
 // within the run; the last block to finish scans the runs' totals. The kernel also checks both
 // inputs (A row by row as it counts; B in the warps' second loop) and clamps every row range it
-// reads. Row pointers are read as the caller stores them (int32 or int64). A row of C with more
+// reads. Short rows need no bitmap: their columns are sorted across the warp. Row pointers are read as the
+// caller stores them (int32 or int64). A row of C with more
 // than kSmallCap entries sends the plan to the general path.
 #include <algorithm>
 #include <mutex>

@@ -5,10 +5,11 @@
 //  * tiny  : P_i <= 32, one warp, each lane holds one column; duplicates are found with a
 //            warp match, so no shared table is needed;
 //  * warp  : one warp per row, a shared-memory hash table of 128 / 512 / 2048 keys;
-//  * block : one block per row, a shared-memory hash table of 8192 keys;
-//  * window: one persistent block per row, a shared-memory bitmap of up to 2^20 columns.
+//  * micro, merge : one thread per row of at most 8 entries of A, a merge of the B rows;
+//  * block : one block per row, a bitmap of up to 2^18 columns, or a hash table of 8192 keys;
+//  * window: persistent blocks, one row at a time, a shared-memory bitmap of up to 2^20 columns.
 //            Besides nnz(C_i) it records how many columns of C_i fall in each block of
-//            kBlockCols columns, which the numeric pass uses to plan its windows. When B has
+//            kBlockCols columns (or sub-block of kSubCols), which the numeric pass uses to plan its windows. When B has
 //            more than 2^20 columns the bitmap slides over the columns in windows and a
 //            per-entry cursor in global memory remembers where each B row stopped.
 // Hash tables are sized to at least twice the row's upper bound min(P_i, n), so probing

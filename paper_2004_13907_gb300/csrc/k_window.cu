@@ -1,5 +1,7 @@
-// Windowed numeric pass for rows with more entries of C than a block-wide hash table holds,
-// and the column-block split table of B it reads.
+// Windowed numeric pass for rows with more entries of C than a block-wide table holds,
+// and the column-block split table of B it reads: for plans with a windowed row whose bitmap is not
+// stored (column spaces over 2^20 columns, or over the budget) and for the exact fixed-point modes
+// and their FP64 reruns. The others run over a list of windows (k_winteam.cu).
 //
 // The columns of C are cut into blocks of kBlockCols. The symbolic pass counted, for each
 // windowed row, the entries of C_i in every block. The numeric pass takes the blocks of a
