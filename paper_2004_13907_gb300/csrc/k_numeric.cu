@@ -142,7 +142,9 @@ __global__ void __launch_bounds__(256) k_num_tiny(DevCsr A, DevCsr B, const int3
 // -> 207 us (416 with a merge of columns and values).
 constexpr int kMicroWarps = 4;
 constexpr int kMicroStaged = 8;   // mean entries of a row from which they are staged
-__host__ __device__ inline int micro_warp_bytes(int cap, int maxp) { return cap * 8 + maxp * 32; }
+__host__ __device__ constexpr int micro_warp_bytes(int cap, int maxp) { return cap * 8 + maxp * 32; }
+// Entries staged per warp for rows of `mean` entries (at most kMergeMax).
+constexpr int micro_cap(int64_t mean) { return static_cast<int>((32 * mean + 2 * mean + 31) & ~int64_t(31)); }
 
 // The first U products (of the `m` there are, possibly none) of one B row at bv, times av, added at
 // their places in the row of `len` entries at dval. The places of one B row's products differ, so all
@@ -499,10 +501,17 @@ constexpr int kStep = 4;   // products per thread in one step (loads in flight)
 constexpr int64_t kBitmapMaxWidth = int64_t(1) << 22;   // coarse words: 16 KB
 
 // Coarse words a block keeps: none when every row's words fit the table of `cap` words.
-__host__ __device__ inline int bitmap_coarse_words(int64_t width, int cap) {
+__host__ __device__ constexpr int bitmap_coarse_words(int64_t width, int cap) {
   const int64_t words = (width + 31) >> 5;
   return words <= cap ? 0 : static_cast<int>((words + 31) >> 5);
 }
+
+// Shared bytes of a block with `cap` entries of C and word-table words: one level (the words of the column
+// space, which fit), and two with `coarse` coarse words.
+constexpr size_t bitmap_bytes_direct(int cap, int64_t width) {
+  return size_t(cap) * (8 + 2) + size_t((width + 31) / 32) * (4 + 2);
+}
+constexpr size_t bitmap_bytes(int cap, int coarse) { return size_t(cap) * (8 + 4 + 4 + 4 + 2) + size_t(coarse) * 6; }
 
 template <int NT>
 struct BitmapChunk {
@@ -876,10 +885,12 @@ int launch_num_micro(const DevCsr& A, const DevCsr& B, const int32_t* perm, int6
   // Rows of fewer entries are stored from the merge, whose lanes are then close together (A*P of the
   // Galerkin set-up, 3 entries a row: 41 us against 59).
   const int64_t mean = (entries + count - 1) / count;
-  const int cap = static_cast<int>((32 * mean + 2 * mean + 31) & ~int64_t(31));
-  const size_t sm = size_t(kMicroWarps) * micro_warp_bytes(cap, maxp);   // at most 4 x 19,456 bytes
+  const int cap = micro_cap(mean);
+  const size_t sm = size_t(kMicroWarps) * micro_warp_bytes(cap, maxp);
   auto go = [&](auto kernel, size_t smem) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    // (the limit belongs to the kernel: always the most any call needs, so that no thread lowers another's)
+    constexpr int most = kMicroWarps * micro_warp_bytes(micro_cap(kMergeMax), kMergeMax);
+    if (smem) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     kernel<<<grid_rows(count, kMicroWarps * 32, num_sms * 32), kMicroWarps * 32, smem, s>>>(A, B, perm, count, cap, maxp,
                                                                                            c_off, ccol, cval, abase, err);
   };
@@ -919,10 +930,14 @@ int launch_num_block(int log2S, int mode, const DevCsr& A, const DevCsr& B, cons
     const int cap = log2S == 11 ? 1024 : (max_nnz <= 2048 ? 2048 : 4096);
     const int cw = bitmap_coarse_words(width, cap);
     const bool direct = cw == 0 && width <= 65536;
-    const size_t sm = direct ? size_t(cap) * (8 + 2) + size_t((width + 31) / 32) * (4 + 2)
-                             : size_t(cap) * (8 + 4 + 4 + 4 + 2) + size_t(cw) * 6;
+    const size_t sm = direct ? bitmap_bytes_direct(cap, width) : bitmap_bytes(cap, cw);
     auto go = [&](auto kernel) {
-      if (sm > 40 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+      // (the limit belongs to the kernel: always the most any call needs, so that no thread lowers another's)
+      constexpr int kMost = 4096;
+      constexpr size_t direct_most = bitmap_bytes_direct(kMost, 65536);
+      constexpr size_t most = bitmap_bytes(kMost, bitmap_coarse_words(kBitmapMaxWidth, 0));
+      if (sm > 40 * 1024)
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(direct ? direct_most : most));
       kernel<<<grid_rows(count, 1, num_sms * 16), 256, sm, s>>>(A, B, perm, count, c_off, ccol, cval, abase, awidth, width,
                                                                cap, row_flag, negflag, err);
     };

@@ -470,8 +470,10 @@ int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int
   cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
   const int64_t cols = width < kSymWinBits ? width : kSymWinBits;
   const int words = static_cast<int>((cols + kBlockCols - 1) / kBlockCols * kBlockWords);
-  auto go = [&](auto kernel, int threads, int blocks) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * words);
+  // (the limit belongs to the kernel, not to the call: always the most any call needs, as another thread may
+  // be about to launch the kernel with more than this call's share)
+  auto go = [&](auto kernel, int threads, int blocks, int most_words) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * most_words);
     const int64_t g = count < int64_t(num_sms) * blocks ? count : int64_t(num_sms) * blocks;
     kernel<<<static_cast<unsigned>(g), threads, 4 * words, s>>>(A, B, words, perm, count, counter, nnz_row, win_slot,
                                                                 blockcnt, nblocks, sub, cursor, abase, awidth, width,
@@ -484,9 +486,9 @@ int launch_sym_window(const DevCsr& A, const DevCsr& B, const int32_t* perm, int
   // A single row that outweighs an SM's share of the products keeps the larger block, as its block
   // finishes last.
   const int64_t share = 2 * total_products / num_sms;
-  if (words <= kSymWinWords6 && max_row_products * 6 <= share) go(k_sym_window<256, 6>, 256, 6);
-  else if (words <= kSymWinWords3 && max_row_products * 3 <= share) go(k_sym_window<512, 3>, 512, 3);
-  else go(k_sym_window<kSymWinThreads, 1>, kSymWinThreads, 1);
+  if (words <= kSymWinWords6 && max_row_products * 6 <= share) go(k_sym_window<256, 6>, 256, 6, kSymWinWords6);
+  else if (words <= kSymWinWords3 && max_row_products * 3 <= share) go(k_sym_window<512, 3>, 512, 3, kSymWinWords3);
+  else go(k_sym_window<kSymWinThreads, 1>, kSymWinThreads, 1, kSymWinBits / 32);
   return 1;
 }
 
