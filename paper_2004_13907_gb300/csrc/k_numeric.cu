@@ -15,6 +15,8 @@
 //  * window: rows with more entries than a block table (k_winteam.cu, k_window.cu).
 // Sums are accumulated with shared-memory FP64 atomics, so their order (and the last bits of
 // a value) can change from run to run; the pattern is always exact.
+#include <type_traits>
+
 #include "enumerate.cuh"
 
 namespace spg {
@@ -496,6 +498,19 @@ __global__ void __launch_bounds__(256) k_num_warp(DevCsr A, DevCsr B, const int3
 // and bitonic sort -> bitmaps: 20,000^2 uniform (19,400 rows of 1,540 entries) 3.83 -> 0.36 ms,
 // R-MAT 2^17 2.67 -> 0.46 ms, R-MAT 2^19 7.87 -> 1.19 ms. Columns stored by the products (Direct): 20,000^2
 // 0.355 -> 0.30 ms.
+//
+// Rows of many products per entry are bound by the enumerations, two or three of them, where the hash table needs
+// one. A class of such rows by its mean (kManyProducts) takes instances of its own (Many), whose rows find
+// their first and last column, from the ends of their B rows. Within `span` columns a row adds each product
+// at its column, in one enumeration, and a byte per column says which were reached; else its words are
+// numbered from its first column on, so that a band of a wide column space needs one level only. Numeric
+// pass, ms, hash table / ranks / this: 30,000 rows of 1,000 entries in bands of a 300,000 column space, 8
+// products per entry 2.91, 3.13, 1.35, 124 per entry 18.3, 39.4, 16.3; 70,000 rows of all 1,000 columns, 85
+// per entry 31.5, 36.1, 28.3. 20,000 rows of 900 scattered columns of 300,000, 35 per entry: 10.6, 5.7, 6.0 (two
+// levels). In FP32 the table's scattered rows are as fast from about 32 per entry on (5.97, 5.88; 14.2 and 15.7
+// with 100): two levels hash from there.
+constexpr int kManyProducts = 4, kManyProductsF32 = 32;
+constexpr int kSpan = 4096;
 constexpr int kHeld = 8;   // products per thread held in registers
 constexpr int kStep = 4;   // products per thread in one step (loads in flight)
 constexpr int64_t kBitmapMaxWidth = int64_t(1) << 22;   // coarse words: 16 KB
@@ -508,10 +523,13 @@ __host__ __device__ constexpr int bitmap_coarse_words(int64_t width, int cap) {
 
 // Shared bytes of a block with `cap` entries of C and word-table words: one level (the words of the column
 // space, which fit), and two with `coarse` coarse words.
-constexpr size_t bitmap_bytes_direct(int cap, int64_t width) {
-  return size_t(cap) * (8 + 2) + size_t((width + 31) / 32) * (4 + 2);
+// With `span`, room for a sum and a byte per column of that many.
+constexpr size_t bitmap_bytes_direct(int cap, int64_t width, int span) {
+  return size_t(cap > span ? cap : span) * 8 + size_t(cap) * 2 + size_t((width + 31) / 32) * (4 + 2) + span;
 }
-constexpr size_t bitmap_bytes(int cap, int coarse) { return size_t(cap) * (8 + 4 + 4 + 4 + 2) + size_t(coarse) * 6; }
+constexpr size_t bitmap_bytes(int cap, int coarse, int span) {
+  return size_t(2 * cap > span ? 2 * cap : span) * 8 + size_t(cap) * (4 + 2) + size_t(coarse) * 6 + span;
+}
 
 template <int NT>
 struct BitmapChunk {
@@ -629,27 +647,31 @@ __device__ __forceinline__ void add_held(double* slot, double held) {
 }
 
 // Direct: every word of the column space fits the table, and a column 16 bits, so that a product stores
-// its column at its rank and no pass walks the bits.
-template <int NT, int Mode, bool Direct>
+// its column at its rank and no pass walks the bits. Many: rows of many products per entry look for their
+// ends (span > 0).
+template <int NT, int Mode, bool Direct, bool Many>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B, const int32_t* __restrict__ perm,
                                                      int64_t count, const int64_t* __restrict__ c_off,
                                                      int32_t* __restrict__ ccol, void* __restrict__ cval,
                                                      const int32_t* __restrict__ abase,
                                                      const int32_t* __restrict__ awidth, int64_t width_all, int cap,
-                                                     int32_t* __restrict__ row_flag,
+                                                     int span, int32_t* __restrict__ row_flag,
                                                      const int32_t* __restrict__ negflag, uint32_t* err) {
   extern __shared__ double smem_f64[];
   __shared__ BitmapChunk<NT> ck;
-  double* vals = smem_f64;                                          // [cap], by rank
+  __shared__ uint32_t s_ends[2];                                    // a row's first and last column
+  double* vals = smem_f64;                                          // [cap] by rank, or [span] by column
   const int table = Direct ? (static_cast<int>(width_all) + 31) >> 5 : cap;   // words of the word table
   const int coarse_all = Direct ? 0 : bitmap_coarse_words(width_all, cap);
-  uint32_t* fine = reinterpret_cast<uint32_t*>(vals + cap);         // [table], the word table (zero between rows)
-  uint32_t* coarse = fine + table;                                  // a bit per word (zero between rows)
-  int32_t* gword = reinterpret_cast<int32_t*>(coarse + coarse_all); // [cap], two levels: word number of a table word
+  int32_t* gword = reinterpret_cast<int32_t*>(vals + cap);          // [cap], two levels: word number of a table word
   int32_t* colbuf = gword + cap;                                    // [cap], two levels: the columns by rank
-  uint16_t* fpre = reinterpret_cast<uint16_t*>(Direct ? gword : colbuf + cap);   // [table]
+  uint32_t* fine = reinterpret_cast<uint32_t*>(vals + max(Direct ? cap : 2 * cap, span));   // [table], the word
+                                                                    //   table (zero between rows)
+  uint32_t* coarse = fine + table;                                  // a bit per word (zero between rows)
+  uint16_t* fpre = reinterpret_cast<uint16_t*>(coarse + coarse_all);   // [table]
   uint16_t* cpre = fpre + table;                                    // [coarse_all]
   uint16_t* cols = cpre;                                            // [cap], Direct: the columns by rank
+  uint8_t* reached = reinterpret_cast<uint8_t*>(Direct ? cols + cap : cpre + coarse_all);   // [span], by column
   for (int t = threadIdx.x; t < table + coarse_all; t += NT) fine[t] = 0u;
   for (int64_t r = blockIdx.x; r < count; r += gridDim.x) {
     const int32_t i = perm[r];
@@ -657,12 +679,18 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
     const int64_t na = A.rp[i + 1] - a0;
     const int64_t off = c_off[i];
     const int64_t len = c_off[i + 1] - off;
-    const int32_t cb = abase ? abase[i] : 0;   // the row's columns are [cb, cb + width)
-    const uint32_t width = static_cast<uint32_t>(awidth ? awidth[i] : width_all);
-    const int words = static_cast<int>((width + 31) >> 5);
-    const bool direct = Direct || words <= cap;   // (a narrower job of a batch may fit where the widest does not)
+    int32_t cb = abase ? abase[i] : 0;   // the row's columns are [cb, cb + width)
+    uint32_t width = static_cast<uint32_t>(awidth ? awidth[i] : width_all);
+    int words = static_cast<int>((width + 31) >> 5);
+    bool direct = Direct || words <= cap;   // (a narrower job of a batch may fit where the widest does not)
+    int32_t first = 0;                      // the column of the row's space at cb
+    bool by_column = false;
     if (Mode == kModeF32C && threadIdx.x == 0 && !f32c_hash_row_ok(negflag, na)) row_flag[i] = 1;
-    __syncthreads();   // the previous row's clearing of the bitmaps
+    if (Many && threadIdx.x == 0) {
+      s_ends[0] = 0xffffffffu;
+      s_ends[1] = 0u;
+    }
+    __syncthreads();   // (also: the previous row's clearing of the bitmaps)
     // the table word of column rel (two levels), -1 past the table (a row counted otherwise)
     auto table_word = [&](uint32_t rel) {
       const uint32_t cw = coarse[rel >> 10];
@@ -677,6 +705,62 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
     for (int64_t base = 0; base < na; base += NT) {
       bitmap_chunk<NT, Mode>(A, B, a0, na, base, ck);
       keep = na <= NT && ck.ctl[1] <= NT * kHeld;
+      if (Many && base == 0 && !keep) {
+        uint32_t lo = 0xffffffffu, hi = 0u;
+        for (int64_t e = threadIdx.x; e < na; e += NT) {
+          const int32_t k = A.col[a0 + e];
+          const int64_t s = B.rp[k], t = B.rp[k + 1];
+          if (s < t) {
+            lo = min(lo, static_cast<uint32_t>(B.col[s] - cb));
+            hi = max(hi, static_cast<uint32_t>(B.col[t - 1] - cb));
+          }
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if ((threadIdx.x & 31) == 0) {
+          atomicMin(&s_ends[0], lo);
+          atomicMax(&s_ends[1], hi);
+        }
+        __syncthreads();
+        lo = s_ends[0] & ~31u;
+        hi = s_ends[1];
+        if (lo <= hi && hi < width) {   // (else a column outside the row's space: reported below)
+          first = static_cast<int32_t>(lo);
+          cb += first;
+          width = hi - lo + 1;
+          words = static_cast<int>((width + 31) >> 5);
+          direct = Direct || words <= cap;
+          by_column = width <= static_cast<uint32_t>(span);
+        }
+        if (by_column) {
+          for (int t = threadIdx.x; t < words * 32; t += NT) {
+            if (t < span) reached[t] = 0;
+            if (t < static_cast<int>(width)) vals[t] = 0.0;
+          }
+          __syncthreads();
+        }
+      }
+      if (Many && by_column) {
+        bitmap_for_each<NT>(ck, false, [&](int, const int64_t (&j)[kStep], const double (&av)[kStep]) {
+          int32_t c[kStep];
+          double p[kStep];
+#pragma unroll
+          for (int u = 0; u < kStep; ++u) {
+            c[u] = j[u] >= 0 ? B.col[j[u]] : 0;
+            p[u] = j[u] >= 0 ? held_product<Mode>(av[u], value_at<Mode>(B.val, j[u])) : 0.0;
+          }
+#pragma unroll
+          for (int u = 0; u < kStep; ++u) {
+            if (j[u] < 0) continue;
+            const uint32_t rel = static_cast<uint32_t>(c[u] - cb);
+            if (rel >= width) { bad = true; continue; }
+            reached[rel] = 1;
+            add_held<Mode>(&vals[rel], p[u]);
+          }
+        });
+        __syncthreads();
+        continue;
+      }
 #pragma unroll
       for (int u = 0; u < kHeld; ++u) held[u] = -1;
       bitmap_for_each<NT>(ck, keep, [&](int q, const int64_t (&j)[kStep], const double (&av)[kStep]) {
@@ -699,6 +783,29 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
         }
       });
       __syncthreads();
+    }
+    if (Many && by_column) {
+      const int lane = threadIdx.x & 31;
+      for (int w = threadIdx.x >> 5; w < words; w += NT / 32) {
+        const uint32_t t = w * 32 + lane;
+        const unsigned bits = __ballot_sync(0xffffffffu, t < width && reached[t]);
+        if (lane == 0) fine[w] = bits;
+      }
+      __syncthreads();
+      const int cnt = bitmap_prefix<NT>(fine, fpre, words, ck.scan);
+      if (cnt != len) bad = true;
+      for (uint32_t t = threadIdx.x; t < width; t += NT) {
+        const uint32_t bits = fine[t >> 5];
+        const int rk = fpre[t >> 5] + __popc(bits & ((1u << (t & 31)) - 1u));
+        if ((bits >> (t & 31) & 1u) && rk < len) {
+          ccol[off + rk] = first + static_cast<int32_t>(t);
+          store_value<Mode>(cval, off + rk, vals[t]);
+        }
+      }
+      __syncthreads();
+      for (int w = threadIdx.x; w < words; w += NT) fine[w] = 0u;
+      if (bad) set_error(err, kErrCount);
+      continue;
     }
     int nwords = words;
     const int cwords = (words + 31) >> 5;
@@ -787,7 +894,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
       for (int w = threadIdx.x; w < nwords; w += NT) {
         uint32_t m = fine[w];
         if (!m) continue;
-        const int col0 = 32 * (direct ? w : gword[w]);
+        const int col0 = first + 32 * (direct ? w : gword[w]);
         for (int rk = fpre[w]; m; m &= m - 1, ++rk)
           if (rk < n_out) colbuf[rk] = col0 + __ffs(m) - 1;
         fine[w] = 0u;
@@ -797,7 +904,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_num_bitmap(DevCsr A, DevCsr B
       __syncthreads();
     }
     for (int t = threadIdx.x; t < n_out; t += NT) {
-      ccol[off + t] = Direct ? static_cast<int32_t>(cols[t]) : colbuf[t];
+      ccol[off + t] = Direct ? first + static_cast<int32_t>(cols[t]) : colbuf[t];
       store_value<Mode>(cval, off + t, vals[t]);
     }
     if (bad) set_error(err, kErrCount);
@@ -921,28 +1028,36 @@ int launch_num_warp(int log2S, int mode, const DevCsr& A, const DevCsr& B, const
 
 int launch_num_block(int log2S, int mode, const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
                      const int64_t* c_off, int32_t* ccol, void* cval, const int32_t* abase, const int32_t* awidth,
-                     int64_t width, int max_nnz, int32_t* row_flag, const int32_t* negflag, uint32_t* err,
-                     int num_sms, cudaStream_t s) {
+                     int64_t width, int max_nnz, int64_t products, int64_t entries, int32_t* row_flag,
+                     const int32_t* negflag, uint32_t* err, int num_sms, cudaStream_t s) {
   if (count <= 0) return 0;
   const bool f32c = mode == kModeF32C;
-  // the coarse bitmap of wider rows would not leave room for four rows on an SM: they hash
-  if (width <= kBitmapMaxWidth) {
-    const int cap = log2S == 11 ? 1024 : (max_nnz <= 2048 ? 2048 : 4096);
-    const int cw = bitmap_coarse_words(width, cap);
+  const int cap = log2S == 11 ? 1024 : (max_nnz <= 2048 ? 2048 : 4096);
+  const int cw = bitmap_coarse_words(width, cap);
+  // (two levels: as many columns as their tables by rank leave room for)
+  const int span = products < kManyProducts * entries ? 0 : (cw == 0 ? kSpan : min(kSpan, 2 * cap));
+  // the coarse bitmap of wider rows would not leave room for four rows on an SM: they hash. So do FP32
+  // rows of two levels and many products
+  if (width <= kBitmapMaxWidth && !(f32c && cw > 0 && products >= kManyProductsF32 * entries)) {
     const bool direct = cw == 0 && width <= 65536;
-    const size_t sm = direct ? bitmap_bytes_direct(cap, width) : bitmap_bytes(cap, cw);
+    const size_t sm = direct ? bitmap_bytes_direct(cap, width, span) : bitmap_bytes(cap, cw, span);
     auto go = [&](auto kernel) {
       // (the limit belongs to the kernel: always the most any call needs, so that no thread lowers another's)
       constexpr int kMost = 4096;
-      constexpr size_t direct_most = bitmap_bytes_direct(kMost, 65536);
-      constexpr size_t most = bitmap_bytes(kMost, bitmap_coarse_words(kBitmapMaxWidth, 0));
+      constexpr size_t direct_most = bitmap_bytes_direct(kMost, 65536, kSpan);
+      constexpr size_t most = bitmap_bytes(kMost, bitmap_coarse_words(kBitmapMaxWidth, 0), kSpan);
       if (sm > 40 * 1024)
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(direct ? direct_most : most));
       kernel<<<grid_rows(count, 1, num_sms * 16), 256, sm, s>>>(A, B, perm, count, c_off, ccol, cval, abase, awidth, width,
-                                                               cap, row_flag, negflag, err);
+                                                               cap, span, row_flag, negflag, err);
     };
-    if (direct) f32c ? go(k_num_bitmap<256, kModeF32C, true>) : go(k_num_bitmap<256, kModeF64, true>);
-    else f32c ? go(k_num_bitmap<256, kModeF32C, false>) : go(k_num_bitmap<256, kModeF64, false>);
+    auto instance = [&](auto many) {
+      constexpr bool kMany = decltype(many)::value;
+      if (direct) f32c ? go(k_num_bitmap<256, kModeF32C, true, kMany>) : go(k_num_bitmap<256, kModeF64, true, kMany>);
+      else f32c ? go(k_num_bitmap<256, kModeF32C, false, kMany>) : go(k_num_bitmap<256, kModeF64, false, kMany>);
+    };
+    if (span > 0) instance(std::true_type{});
+    else instance(std::false_type{});
     return 1;
   }
   const size_t sm = (size_t(1) << log2S) * 12;

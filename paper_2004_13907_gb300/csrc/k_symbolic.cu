@@ -197,20 +197,28 @@ constexpr int kSymWinWords3 = 1 << 14;
 // step per warp (all of them, unless the width itself is below block_max) stay in registers and clear
 // their words afterwards. The hash table it replaces cleared 8,192 slots a row and probed: 20,000^2
 // uniform (d = 2e-3, 19,000 rows of 1,600 products) 231 -> 145 us.
+//
+// A row whose products do not stay in registers sets a byte per column with a plain store where the column
+// space has at most kSymByteCols (its products reach few columns many times: 32 of a warp meet in a few
+// bitmap words, and their atomics wait for one another), and counts the bytes. 30,000 rows of 100,000 products in
+// 1,200 columns: hash table 6.19 ms, bits 6.87, bytes 5.39; 2,040 columns 9.54, 9.60, 7.10.
 constexpr int kSymBitmapCols = kSymWinWords6 * 32;
-template <int NT, int Blocks>
+constexpr int kSymByteCols = 4096;
+template <int NT, int Blocks, bool Bytes>
 __global__ void __launch_bounds__(NT, Blocks) k_sym_bitmap(DevCsr A, DevCsr B, int bitmap_words,
                                                            const int32_t* __restrict__ perm, int64_t count,
                                                            int32_t* __restrict__ nnz_row,
                                                            const int32_t* __restrict__ abase, uint32_t* err) {
-  extern __shared__ uint32_t bm[];  // bitmap_words
+  extern __shared__ uint32_t bm[];  // bitmap_words, and with Bytes a byte per column
   __shared__ int32_t s_excl[NT + 1];
   __shared__ int64_t s_bs[NT];
   __shared__ long long s_scan64[33];
   __shared__ int32_t s_ctl[2];
   __shared__ int32_t s_cnt[2];
   constexpr int kHold = 8;
-  for (int t = threadIdx.x; t < bitmap_words; t += NT) bm[t] = 0u;
+  uint32_t* const bytes = bm + bitmap_words;
+  const int byte_words = Bytes ? 8 * bitmap_words : 0;
+  for (int t = threadIdx.x; t < bitmap_words + byte_words; t += NT) bm[t] = 0u;
   if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
   __syncthreads();
   const uint32_t span = static_cast<uint32_t>(bitmap_words) * 32u;
@@ -226,6 +234,14 @@ __global__ void __launch_bounds__(NT, Blocks) k_sym_bitmap(DevCsr A, DevCsr B, i
     block_range_for_each_product<NT, kHold>(A, B, a0, na, s_excl, s_bs, s_scan64, s_ctl, [&](const int64_t (&j)[kHold]) {
 #pragma unroll
       for (int u = 0; u < kHold; ++u) held[u] = j[u] >= 0 ? static_cast<uint32_t>(B.col[j[u]] - cb) : 0xffffffffu;
+      if (Bytes && (na > NT || s_ctl[1] > NT * kHold)) {
+#pragma unroll
+        for (int u = 0; u < kHold; ++u) {
+          if (held[u] < span) reinterpret_cast<uint8_t*>(bytes)[held[u]] = 1;
+          else outside |= j[u] >= 0;
+        }
+        return;
+      }
 #pragma unroll
       for (int u = 0; u < kHold; ++u) {
         if (held[u] < span) {
@@ -245,6 +261,11 @@ __global__ void __launch_bounds__(NT, Blocks) k_sym_bitmap(DevCsr A, DevCsr B, i
 #pragma unroll
         for (int u = 0; u < kHold; ++u)
           if (held[u] < span) bm[held[u] >> 5] = 0u;
+    } else if (Bytes) {
+      for (int t = threadIdx.x; t < byte_words; t += NT) {
+        cnt += __popc(bytes[t]);
+        bytes[t] = 0u;
+      }
     } else {
       for (int t = threadIdx.x; t < bitmap_words; t += NT) bm[t] = 0u;
     }
@@ -450,8 +471,11 @@ int launch_sym_block(const DevCsr& A, const DevCsr& B, const int32_t* perm, int6
   if (count <= 0) return 0;
   if (width <= kSymBitmapCols) {
     const int words = static_cast<int>((width + 31) / 32);
-    k_sym_bitmap<256, 6><<<grid_rows(count, 1, num_sms * 6), 256, 4 * words, s>>>(A, B, words, perm, count, nnz_row,
-                                                                                abase, err);
+    auto go = [&](auto kernel, int bytes) {
+      kernel<<<grid_rows(count, 1, num_sms * 6), 256, 4 * words + bytes, s>>>(A, B, words, perm, count, nnz_row, abase, err);
+    };
+    if (width <= kSymByteCols) go(k_sym_bitmap<256, 6, true>, 32 * words);
+    else go(k_sym_bitmap<256, 6, false>, 0);
   } else {
     constexpr int kLog2 = 13;
     k_sym_block<kLog2, 512><<<grid_rows(count, 1, num_sms * 8), 512, size_t(4) << kLog2, s>>>(A, B, perm, count,

@@ -152,8 +152,8 @@ int launch_num_warp(int log2S, int mode, const DevCsr& A, const DevCsr& B, const
                     const int32_t* negflag, uint32_t* err, int num_sms, cudaStream_t s);
 int launch_num_block(int log2S, int mode, const DevCsr& A, const DevCsr& B, const int32_t* perm, int64_t count,
                      const int64_t* c_off, int32_t* ccol, void* cval, const int32_t* abase, const int32_t* awidth,
-                     int64_t width, int max_nnz, int32_t* row_flag, const int32_t* negflag, uint32_t* err,
-                     int num_sms, cudaStream_t s);
+                     int64_t width, int max_nnz, int64_t products, int64_t entries, int32_t* row_flag,
+                     const int32_t* negflag, uint32_t* err, int num_sms, cudaStream_t s);
 
 // ---- windowed numeric pass and the column-block split table of B (k_window.cu)
 // Columns of C for the windowed rows with a stored bitmap (k_window.cu); rows without one get

@@ -715,10 +715,13 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
       int32_t* flag = f32c ? p->rerun_flag : nullptr;
       const int32_t* neg = f32c ? p->counters + 8 : nullptr;
       stage_begin(p, SPGEMM_STAGE_NUM_BLOCK, s);
-      nl = launch_num_block(13, mode, p->A, p->B, seg(kNumBlock2), cnt(kNumBlock2), p->c_off, C->col, C->val,
-                            p->abase, p->awidth, p->width, p->cp.block_max, flag, neg, err, p->num_sms, s);
-      nl += launch_num_block(11, mode, p->A, p->B, seg(kNumBlock1), cnt(kNumBlock1), p->c_off, C->col, C->val,
-                             p->abase, p->awidth, p->width, p->cp.block_max, flag, neg, err, p->num_sms, s);
+      auto block = [&](int log2S, int c) {
+        return launch_num_block(log2S, mode, p->A, p->B, seg(c), cnt(c), p->c_off, C->col, C->val, p->abase, p->awidth,
+                                p->width, p->cp.block_max, static_cast<int64_t>(p->cls_sums[c][0]),
+                                static_cast<int64_t>(p->cls_sums[c][2]), flag, neg, err, p->num_sms, s);
+      };
+      nl = block(13, kNumBlock2);
+      nl += block(11, kNumBlock1);
       stage_end(p, SPGEMM_STAGE_NUM_BLOCK, nl, s);
       stage_begin(p, SPGEMM_STAGE_NUM_WARP, s);
       nl = launch_num_warp(10, mode, p->A, p->B, seg(kNumWarp3), cnt(kNumWarp3), p->c_off, C->col, C->val, p->abase,
