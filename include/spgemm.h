@@ -342,8 +342,9 @@ spgemm_status spgemm_autotune_batch(int64_t n_jobs, const spgemm_csr_in* A, cons
  * and nnz are set on return. Rows of T list their entries in ascending column (the order of M's
  * rows). Scratch (about 24 bytes per entry) comes from `alloc` (NULL: the library pool) on
  * `stream` and is freed before return; the call waits for `stream`. Errors: INVALID_ARG (NULL
- * arrays, bad value_bytes), INVALID_CSR (a column of M outside [0, M.cols)), UNSUPPORTED
- * (nnz >= 2^32), INDEX_OVERFLOW (int32 row_ptr too small).
+ * arrays, bad value_bytes), INVALID_CSR (a column of M outside [0, M.cols), or row pointers of M
+ * that decrease, lie outside [0, nnz] or do not run from 0 to nnz), UNSUPPORTED (nnz >= 2^32),
+ * INDEX_OVERFLOW (int32 row_ptr too small).
  *
  * spgemm_coo_to_csr: canonical CSR from nnz (row, col, val) triples in any order (device arrays,
  * int32 indices, values of value_bytes bytes). C: caller-allocated, row_ptr[rows + 1], col/val[nnz];

@@ -246,7 +246,7 @@ int bits_for(int64_t v) {
 }
 
 // Row index of every stored entry of M: a row of up to 8 entries by its thread, a longer one by the
-// whole warp. Row pointers outside [0, nnz] are clamped (and reported).
+// whole warp. Row pointers that decrease, lie outside [0, nnz] or leave an entry to no row are reported.
 __global__ void __launch_bounds__(256) k_expand_rows(const void* __restrict__ rp, int rp64, int64_t m, int64_t nnz,
                                                      uint32_t* __restrict__ row_of, uint32_t* err) {
   const int lane = threadIdx.x & 31;
@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(256) k_expand_rows(const void* __restrict__ rp
     if (i < m) {
       s = at(i);
       e = at(i + 1);
+      if ((i == 0 && s != 0) || (i == m - 1 && e != nnz)) atomicOr(err, kErrInvalidCsr);
       if (s < 0 || e < s || e > nnz) {
         atomicOr(err, kErrInvalidCsr);
         s = e = 0;
@@ -349,7 +350,8 @@ spgemm_status finish(Scratch& sc, uint32_t* err, cudaStream_t s, const char* wha
   sc.ws.release_all();
   if (st != SPGEMM_OK) return st;
   if (h & kErrInvalidCsr)
-    return set_error_msg(SPGEMM_ERR_INVALID_CSR, "%s: an index is out of range or a (row, column) pair repeats", what);
+    return set_error_msg(SPGEMM_ERR_INVALID_CSR,
+                         "%s: an index or row pointer is out of range or a (row, column) pair repeats", what);
   if (h) return set_error_msg(SPGEMM_ERR_INTERNAL, "%s: device check failed (0x%x)", what, h);
   return SPGEMM_OK;
 }
@@ -381,6 +383,7 @@ extern "C" spgemm_status spgemm_csr_transpose(const spgemm_csr_in* M, int32_t va
   if (!T->row_ptr || (nnz > 0 && (!T->col || !T->val)))
     return set_error_msg(SPGEMM_ERR_INVALID_ARG, "T's arrays are NULL");
   if (!T->idx64_rowptr && nnz > 0x7fffffffLL) return set_error_msg(SPGEMM_ERR_INDEX_OVERFLOW, "T needs an int64 row_ptr");
+  if (m == 0 && nnz > 0) return set_error_msg(SPGEMM_ERR_INVALID_CSR, "transposing: entries but no rows");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Scratch sc;
   init_scratch(sc, alloc, stream);
@@ -398,7 +401,7 @@ extern "C" spgemm_status spgemm_csr_transpose(const spgemm_csr_in* M, int32_t va
   cudaMemsetAsync(err, 0, sizeof(uint32_t), s);
   int sorted = 0;
   if (nnz > 0) {
-    if (m > 0) k_expand_rows<<<grid_for(m), 256, 0, s>>>(M->row_ptr, M->idx64_rowptr, m, nnz, row_of, err);
+    k_expand_rows<<<grid_for(m), 256, 0, s>>>(M->row_ptr, M->idx64_rowptr, m, nnz, row_of, err);
     sorted = stable_sort<uint32_t>(ColKeys{M->col, n}, keys, idx, nnz, bits_for(n), hist, tot, err, s);
     k_gather_entries<<<grid_for(nnz), 256, 0, s>>>(idx[sorted], nnz, row_of, M->val, vbytes, T->col, T->val);
   }
