@@ -622,11 +622,13 @@ __global__ void __launch_bounds__(kTeam * 32, kTeamBlocks) k_num_winteam(
 }  // namespace
 
 int64_t win_list_bytes(int64_t rows, int64_t entries, int64_t nsub, int32_t merge_cap, int f32c, int64_t* cap) {
-  // a window ends by its span or the end of a run of 64 sub-blocks, or it and the next hold more than
-  // merge_cap entries together; and it holds at least one sub-block
+  // a window ends with its run of 64 sub-blocks, or it and the next of the run hold more than merge_cap
+  // entries together (a run of e entries: at most 2 e / merge_cap + 1 windows); and it holds at least one
+  // sub-block
+  static_assert(kWinSpan >= 64, "the span of a window does not end it inside a run");
   const int64_t most = f32c ? kWideCap : kWinCap;
   const int64_t m = merge_cap < 1 ? 1 : (merge_cap < most ? merge_cap : most);
-  const int64_t by_entries = 2 * (entries / m + 1) + rows * ((nsub + 63) / 64 + nsub / kWinSpan + 1);
+  const int64_t by_entries = 2 * (entries / m + 1) + rows * ((nsub + 63) / 64);
   *cap = by_entries < rows * nsub ? by_entries : rows * nsub;
   return *cap * static_cast<int64_t>(sizeof(WinRecord));
 }

@@ -524,6 +524,7 @@ int64_t window_list_cap(const spgemm_plan_s* p, int64_t nwin) {
   return cap < kListCapMax ? cap : kListCapMax;
 }
 
+// List of the windows of any `nwin` windowed rows.
 int64_t window_list_bytes(const spgemm_plan_s* p, int64_t nwin, int64_t* cap) {
   unsigned long long entries = 0;
   for (int c = kNumWin0; c <= kNumWin3; ++c) entries += p->cls_sums[c][2];
@@ -539,6 +540,18 @@ int numeric_windows(spgemm_plan_s* p, const int32_t* perm, int64_t nwin, int64_t
                     cudaStream_t s) {
   if (nwin <= 0) return 0;
   int nl = 0;
+  bool listed = p->wins != nullptr;
+  if (!listed) {
+    // one list of all windows; where there is no room for it, a list for as many rows at a time as there is
+    p->wins_rows = nwin;
+    for (;;) {
+      const int64_t bytes = window_list_bytes(p, p->wins_rows, &p->wins_cap);
+      p->wins = p->ws.get(static_cast<size_t>(bytes));
+      if (p->wins) break;
+      if (p->wins_rows == 1) return -1;
+      p->wins_rows = (p->wins_rows + 1) / 2;
+    }
+  }
   if (!p->split_tried) {
     // split table of B, once per plan, when it fits the budget (else the kernel searches)
     p->split_tried = true;
@@ -550,19 +563,17 @@ int numeric_windows(spgemm_plan_s* p, const int32_t* perm, int64_t nwin, int64_t
   }
   const bool f32c = p->prec == SPGEMM_F32_COMPENSATED;
   const int32_t* neg = f32c ? p->counters + 8 : nullptr;
-  const bool listed = p->wins != nullptr;
-  if (!listed) {
-    const int64_t bytes = window_list_bytes(p, nwin, &p->wins_cap);
-    p->wins = p->ws.get(static_cast<size_t>(bytes));
-    if (!p->wins) return -1;
+  listed = listed && p->wins_rows >= nwin && !f32c;
+  for (int64_t r = 0; r < nwin; r += p->wins_rows) {
+    if (!listed)
+      nl += launch_win_plan(p->A, perm + r, nwin - r < p->wins_rows ? nwin - r : p->wins_rows, p->win_slot, nslots,
+                            p->blockcnt, p->nblocks, p->opts.window_hash_fill, p->c_off, p->woff, p->abase, p->awidth,
+                            p->width, neg, p->wins, p->wins_cap, p->counters + 9, p->num_sms, &p->summary->err, s);
+    nl += launch_num_winteam(p->A, p->B, p->wins, p->counters + 9, p->wins_cap, p->counters + 1, p->blockcnt, p->nblocks,
+                             p->split_sub, C->col, C->val, p->wbits, neg, f32c ? p->rerun_flag : nullptr, p->num_sms,
+                             &p->summary->err, s);
   }
-  if (!listed || f32c)
-    nl += launch_win_plan(p->A, perm, nwin, p->win_slot, nslots, p->blockcnt, p->nblocks, p->opts.window_hash_fill,
-                          p->c_off, p->woff, p->abase, p->awidth, p->width, neg, p->wins, p->wins_cap,
-                          p->counters + 9, p->num_sms, &p->summary->err, s);
-  return nl + launch_num_winteam(p->A, p->B, p->wins, p->counters + 9, p->wins_cap, p->counters + 1, p->blockcnt,
-                                 p->nblocks, p->split_sub, C->col, C->val, p->wbits, neg, f32c ? p->rerun_flag : nullptr,
-                                 p->num_sms, &p->summary->err, s);
+  return nl;
 }
 
 }  // namespace
@@ -662,7 +673,8 @@ spgemm_status numeric_run(spgemm_plan_s* p, spgemm_csr_out* C, cudaStream_t s) {
                                                      p->num_sms, s);
     if (p->sub) {
       const int n = numeric_windows(p, seg(kNumWin0), nwin, nslots, C, s);
-      if (n < 0) return set_error_msg(SPGEMM_ERR_OOM, "device workspace allocation of the window list failed");
+      if (n < 0) return set_error_msg(SPGEMM_ERR_OOM, "device workspace allocation of the window list failed "
+                                                           "(window_cols_max_mb 0 needs none)");
       nl += n;
     }
     if (!p->sub && nwin > 0 && !p->split_tried) {

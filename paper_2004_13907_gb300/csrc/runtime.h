@@ -56,8 +56,8 @@ struct spgemm_plan_s {
   int64_t nblocks = 0;               // column blocks, or sub-blocks (sub), of the widest row
   bool sub = false;                  // every windowed row has a stored bitmap: the pass over a list of windows
   uint32_t* split_sub = nullptr;     // sub: split table of B by sub-blocks
-  void* wins = nullptr;              // sub: the list of windows (counters[9] of them)
-  int64_t wins_cap = 0;
+  void* wins = nullptr;              // sub: the list of windows (counters[9] of them) of up to
+  int64_t wins_cap = 0, wins_rows = 0;   // wins_rows rows, with room for wins_cap
   int32_t* cursor = nullptr;
   int32_t* split = nullptr;          // column-block split table of B (windowed numeric rows)
   uint32_t* wbits = nullptr;         // column bitmaps of windowed rows, stored by the symbolic pass
