@@ -645,9 +645,9 @@ int launch_rowptr_to64(const int32_t* in, int64_t* out, int64_t n1, cudaStream_t
 }
 
 int launch_validate(const void* rp, int rp64, int64_t rows, int64_t cols, int64_t nnz, const int32_t* col,
-                    int64_t* rp_out, uint32_t* err, cudaStream_t s) {
+                    int64_t* rp_out, uint32_t* err, int num_sms, cudaStream_t s) {
   // every block the same number of kCheckEntries, one wave of them; few entries: the rows' share
-  const int64_t pieces = (nnz + kCheckEntries - 1) / kCheckEntries, most = 152 * kCheckBlocks;
+  const int64_t pieces = (nnz + kCheckEntries - 1) / kCheckEntries, most = int64_t(num_sms) * kCheckBlocks;
   const int64_t per = pieces > most ? (pieces + most - 1) / most : 1;
   int64_t g = pieces > 0 ? (pieces + per - 1) / per : 1;
   const int64_t by_rows = (rows + 255) / 256 < most ? (rows + 255) / 256 : most;
@@ -658,14 +658,14 @@ int launch_validate(const void* rp, int rp64, int64_t rows, int64_t cols, int64_
 
 int launch_count(const CsrArrays& A, const CsrArrays& B, int check, int64_t* a64, ClassParams cp, int64_t* P,
                  int32_t* nnz_row, int32_t* tile_hist, int64_t* tile_sum, int64_t* tile_max, uint32_t* err,
-                 cudaStream_t s) {
+                 int num_sms, cudaStream_t s) {
   const int64_t ntiles = (A.rows + kTileRows - 1) / kTileRows;
   if (ntiles == 0) return 0;
   cudaMemsetAsync(tile_hist, 0, sizeof(int32_t) * ntiles * kMaxClasses, s);
   cudaMemsetAsync(tile_sum, 0, sizeof(int64_t) * ntiles, s);
   if (tile_max) cudaMemsetAsync(tile_max, 0, sizeof(int64_t) * ntiles, s);
   int run = 32;
-  while (run > 1 && A.rows < int64_t(run / 2) * 8 * 152 * 8) run /= 2;   // eight blocks per SM or more
+  while (run > 1 && A.rows < int64_t(run / 2) * 8 * num_sms * 8) run /= 2;   // eight blocks per SM or more
   const int64_t blocks = (A.rows + 8 * run - 1) / (8 * run);
   k_count<<<static_cast<unsigned>(blocks), 256, 0, s>>>(A, B, run, check, a64, cp, P, nnz_row, tile_hist, tile_sum, tile_max,
                                                        err);

@@ -647,10 +647,11 @@ int launch_win_plan(const DevCsr& A, const int32_t* perm, int64_t count, const i
   return 1;
 }
 
-int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint32_t* split, cudaStream_t s) {
+int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint32_t* split, int num_sms,
+                      cudaStream_t s) {
   if (B.rows <= 0) return 0;
   int64_t g = (B.rows + kSplitWarps - 1) / kSplitWarps;
-  if (g > 152 * 64) g = 152 * 64;
+  if (g > int64_t(num_sms) * 64) g = int64_t(num_sms) * 64;
   k_bsplit_sub<<<static_cast<unsigned>(g), kSplitWarps * 32, 0, s>>>(B, nsub, bbase, split);
   return 1;
 }

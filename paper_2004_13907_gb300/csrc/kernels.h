@@ -94,12 +94,12 @@ int launch_rowptr_rebase(const void* in, int idx64, int64_t r0, int64_t n1, int6
                          cudaStream_t s);
 // Canonical-CSR check; rp_out (may be null) receives the row pointers as int64.
 int launch_validate(const void* rp, int rp64, int64_t rows, int64_t cols, int64_t nnz, const int32_t* col,
-                    int64_t* rp_out, uint32_t* err, cudaStream_t s);
+                    int64_t* rp_out, uint32_t* err, int num_sms, cudaStream_t s);
 // P_i of every row, its symbolic class, and (check) the canonical-CSR check of A; a64 (may be null)
 // receives A's row pointers as int64.
 int launch_count(const CsrArrays& A, const CsrArrays& B, int check, int64_t* a64, ClassParams cp, int64_t* P,
                  int32_t* nnz_row, int32_t* tile_hist, int64_t* tile_sum, int64_t* tile_max, uint32_t* err,
-                 cudaStream_t s);
+                 int num_sms, cudaStream_t s);
 int launch_class_scan(int64_t ntiles, int nclasses, int32_t* tile_hist, const int64_t* tile_sum,
                        const int64_t* tile_max, int64_t* tile_sum_off, Summary* summary,
                        cudaStream_t s);
@@ -179,7 +179,8 @@ int launch_win_plan(const DevCsr& A, const int32_t* perm, int64_t count, const i
                     const uint16_t* subcnt, int64_t nsub, int32_t merge_cap, const int64_t* c_off, const int64_t* woff,
                     const int32_t* abase, const int32_t* awidth, int64_t width, const int32_t* negflag, void* wins,
                     int64_t cap, int32_t* n_wins, int num_sms, uint32_t* err, cudaStream_t s);
-int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint32_t* split, cudaStream_t s);
+int launch_bsplit_sub(const DevCsr& B, int64_t nsub, const int32_t* bbase, uint32_t* split, int num_sms,
+                      cudaStream_t s);
 int launch_num_winteam(const DevCsr& A, const DevCsr& B, const void* wins, const int32_t* n_wins, int64_t wins_cap,
                        int32_t* counter, const uint16_t* subcnt, int64_t nsub, const uint32_t* split, int32_t* ccol,
                        void* cval, const uint32_t* wbits, const int32_t* negflag, int32_t* row_flag, int num_sms,

@@ -324,9 +324,11 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
     // no wait here: the count pass clamps every access, and the error word is read with the plan's
     // summary below (an invalid input is reported before any other pass runs)
     if (m == 0)
-      conv += launch_validate(A->row_ptr, A->idx64_rowptr, m, A->cols, A->nnz, A->col, nullptr, &p->summary->err, s);
+      conv += launch_validate(A->row_ptr, A->idx64_rowptr, m, A->cols, A->nnz, A->col, nullptr, &p->summary->err,
+                              p->num_sms, s);
     if (!same)
-      conv += launch_validate(B->row_ptr, B->idx64_rowptr, B->rows, n, B->nnz, B->col, b64, &p->summary->err, s);
+      conv += launch_validate(B->row_ptr, B->idx64_rowptr, B->rows, n, B->nnz, B->col, b64, &p->summary->err,
+                              p->num_sms, s);
     if ((st = cuda_status(cudaGetLastError(), "launching validation")) != SPGEMM_OK) return st;
   }
   stage_end(p, SPGEMM_STAGE_VALIDATE, conv, s);
@@ -335,7 +337,7 @@ spgemm_status plan_run(spgemm_plan_s* p, const spgemm_csr_in* A, const spgemm_cs
     const CsrArrays ca{m, A->cols, A->nnz, A->row_ptr, A->idx64_rowptr, A->col};
     const CsrArrays cb{B->rows, n, B->nnz, B->row_ptr, B->idx64_rowptr, B->col};
     int nl = launch_count(ca, cb, o.validate, a64, p->cp, p->P, p->nnz_row, p->tile_hist, p->tile_sum, p->tile_max,
-                          &p->summary->err, s);
+                          &p->summary->err, p->num_sms, s);
     nl += launch_class_scan(p->ntiles, kSymNumClasses, p->tile_hist, p->tile_sum, p->tile_max, nullptr,
                             p->summary, s);
     nl += launch_scatter_sym(p->A, p->cp, p->P, p->tile_hist, p->summary, p->perm_s, s);
@@ -558,7 +560,7 @@ int numeric_windows(spgemm_plan_s* p, const int32_t* perm, int64_t nwin, int64_t
     const int64_t bytes = split_sub_bytes(p);
     if (bytes <= (int64_t(p->opts.window_split_max_mb) << 20)) {
       p->split_sub = static_cast<uint32_t*>(p->ws.get(static_cast<size_t>(bytes) + sizeof(uint32_t)));
-      if (p->split_sub) nl += launch_bsplit_sub(p->B, p->nblocks, p->bbase, p->split_sub, s);
+      if (p->split_sub) nl += launch_bsplit_sub(p->B, p->nblocks, p->bbase, p->split_sub, p->num_sms, s);
     }
   }
   const bool f32c = p->prec == SPGEMM_F32_COMPENSATED;

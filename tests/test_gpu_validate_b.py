@@ -23,8 +23,9 @@ def _gpu():
 class _Check:
     """B with rows of the given lengths, columns 0, 1, ... in each; A is one row that names B's first row."""
 
-    def __init__(self, lens, idx64):
+    def __init__(self, lens, idx64, **opts):
         import paper_2004_13907_gb300 as sp
+        self.opts = opts
         lens = np.asarray(lens, np.int64)
         self.rows, self.cols = lens.size, int(max(lens.max(initial=0), 4))
         rp = np.concatenate([[0], np.cumsum(lens)])
@@ -47,7 +48,7 @@ class _Check:
     def refused(self, rp=None, col=None):
         import paper_2004_13907_gb300 as sp
         try:
-            sp.spgemm_plan_destroy(self.plan(rp, col))
+            sp.spgemm_plan_destroy(self.plan(rp, col, **self.opts))
         except sp.SpgemmError as e:
             return e.name == "INVALID_CSR"
         return False
@@ -121,6 +122,17 @@ def test_shares_of_several_pieces(idx64):
                  + [pieces + k * PIECE + d for k in range(4) for d in (-1, 0, 1)])
     for r in (225_000, 240_000, M.rows - 3_500):  # inside runs of empty rows
         assert M.with_rp(r, 1) and M.with_rp(r, -1), r
+
+
+@pytest.mark.parametrize("name", ["long", "ones", "ones_among_empty"])
+def test_on_one_sm(name):
+    # six blocks, each with a share of the same number of pieces
+    M = _Check(LENS[name] * 6, False, max_sms=1)
+    assert not M.refused()
+    pieces = -(-M.nnz // PIECE)
+    share = -(-pieces // 6) * PIECE
+    assert share > PIECE
+    M.violations([share - 1, share, share + PIECE - 1, share + PIECE, share + PIECE + 1, 3 * share + PIECE, M.nnz - 1])
 
 
 @pytest.mark.parametrize("where", ["first", "between", "last"])
