@@ -126,8 +126,12 @@ typedef struct spgemm_opts {
                                  them instead of marking every partial product again; rows beyond
                                  the budget are marked again (default 49152; 0: never store) */
   int32_t fp64_accumulate;    /* how FP64 sums are formed (F64 plans):
-                                 0 (default): FP64 shared-memory atomics (fastest; the order of
-                                   the additions, so the last bits, may vary from run to run);
+                                 0 (default): FP64 shared-memory atomics (fastest). The order of
+                                   the additions may vary from run to run, and in rows of the
+                                   windowed path so may whether a product is added fused (one
+                                   rounding) or rounded first: the last bits vary, also those of
+                                   an entry of two products, and products that cancel exactly
+                                   can leave one rounding error of a product instead of zero;
                                  1: rows of the windowed path (more entries of C than a block
                                    table) sum every entry exactly in integer fixed point and round
                                    it once: the correctly rounded sum of the entry's products;

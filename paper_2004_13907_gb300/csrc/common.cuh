@@ -132,6 +132,8 @@ __device__ __forceinline__ void set_error(uint32_t* err, uint32_t code) { atomic
 // numeric pass, ms, with atomicAdd, one try, two (taken), three, compare-and-swap only: R-MAT 2^17 6.31,
 // 5.79, 5.69, 5.68, 6.47; 30,000^2 uniform 4.64, 4.54, 4.53, 4.53, 4.60. Relative error against quadruple
 // precision, atomicAdd and this: 6.2e-17 and 5.5e-17 (uniform), 3.9e-16 both (R-MAT).
+// Which products are fused varies from run to run, so the last bits of an entry of two products can too, and
+// products that cancel exactly when rounded can leave one rounding error.
 __device__ __forceinline__ void add_product_f64(double* sum, double a, double b) {
   unsigned long long* const p = reinterpret_cast<unsigned long long*>(sum);
 #pragma unroll
