@@ -36,7 +36,9 @@ constexpr int kSlots = 4;        // partial products per lane in one step (loads
 constexpr int kRunShared = 512;  // symbolic runs of up to this many rows keep their counts in shared memory
 constexpr int kSymWarpBytes = 4096;       // bitmap bytes per symbolic warp (all its row slots)
 constexpr int kNumSmemMax = 64 * 1024;   // numeric: 4 warps x (192 B x 32 + 10 B x 1,024) = 65,536 B at most
-constexpr double kFewEntries = 8.0, kFewProducts = 16.0;   // k_small_sym: Few, averages per row
+constexpr double kFewEntries = 8.0, kFewProducts = 16.0;   // k_small_sym: Few, averages per row,
+constexpr int kFewPer = 16;                                //   and words of the bitmap per lane at least
+constexpr int32_t kLookEntries = 128;   // k_small_sym: entries of A between two looks at the common flag
 constexpr unsigned kFull = 0xffffffffu;
 enum : uint32_t { kSmallTooLong = 1u };   // summary->small_flags bit: a row needs the general path
 
@@ -360,11 +362,13 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   int64_t prod = 0;
   int max_cnt = 0;
   // A row of C over kSmallCap entries sends the whole product to the general path: the warp that finds
-  // one says so at once, and the others, which look once per group (a load that the group's work hides),
-  // stop there. Counting on to the end took 1.8 ms of a 30,000^2 product whose every row is too long. A row
-  // of many entries of A is looked at after every 32 of them (counting the first row of every warp
-  // to its end: 0.1 ms more).
+  // one says so at once, and the others, which look after every kLookEntries entries of A (a load that the
+  // next group's work hides; all warps look at one word, and a look per group took 65,000 short rows 31 us
+  // instead of 24), stop there. Counting on to the end took 1.8 ms of a 30,000^2 product whose every row is
+  // too long. A row of many entries of A is looked at after every 32 of them (counting the first row of
+  // every warp to its end: 0.1 ms more).
   bool stop = false;
+  int32_t unseen = 0;   // entries of A since the last look
   auto row_counted = [&](int64_t r, int cnt) {
     if (lane == 0) {
       nnz_row[r] = cnt;
@@ -374,6 +378,7 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   };
   auto bitmap_rows = [&](int64_t gs, int ng) {
     const RowGroup gr = group_rows(A, gs, ng, chk, bad);
+    unseen += gr.E;
     // lane g < ng: the first column of row gs + g's column space (a stacked batch's job)
     const int32_t cb_lane = A.cbase && lane < ng ? A.cbase[gs + lane] : 0;
     for (int32_t c0 = 0; c0 < gr.E; c0 += 32) {
@@ -421,6 +426,7 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
   auto sorted_rows = [&](int64_t gs, int ng) {
     const RowGroup gr = group_rows(A, gs, ng, chk, bad);
     if (gr.E > 32) return false;
+    unseen += gr.E;
     const int32_t cb_lane = A.cbase && lane < ng ? A.cbase[gs + lane] : 0;
     int g;
     int64_t bs;
@@ -474,7 +480,11 @@ __global__ void __launch_bounds__(kSymWarps * 32) k_small_sym(SmallCsr A, SmallC
     return true;
   };
   for (int64_t gs = r0 + wid * G; gs < r1 && !stop; gs += int64_t(kSymWarps) * G) {
-    const uint32_t flags = *reinterpret_cast<const volatile uint32_t*>(&sum->small_flags);
+    uint32_t flags = 0;
+    if (unseen >= kLookEntries) {
+      flags = *reinterpret_cast<const volatile uint32_t*>(&sum->small_flags);
+      unseen = 0;
+    }
     const int ng = r1 - gs < G ? static_cast<int>(r1 - gs) : G;
     if constexpr (Few) {
       if (!sorted_rows(gs, ng))
@@ -737,7 +747,10 @@ int per_index(int per) { return __builtin_ctz(static_cast<unsigned>(per)); }
 template <int PER>
 void sym_launch(dim3 g, size_t smem, cudaStream_t s, const SmallCsr& A, const SmallCsr& B, int32_t width, int check,
                 SmallGrid sg, int32_t* nnz_row, int32_t* loc, int64_t* blk, Summary* sum, Summary* hsum) {
-  const auto kernel = sg.few ? k_small_sym<PER, true> : k_small_sym<PER, false>;
+  auto kernel = k_small_sym<PER, false>;
+  if constexpr (PER >= kFewPer) {
+    if (sg.few) kernel = k_small_sym<PER, true>;
+  }
   kernel<<<g, kSymWarps * 32, smem, s>>>(A, B, width, check, sg.run, sg.groups, nnz_row, loc, blk, sum, hsum);
 }
 
@@ -756,15 +769,14 @@ __global__ void __launch_bounds__(256) k_small_offsets(const int32_t* __restrict
     c_off[i] = i < m ? blk[i / run] + loc[i] : blk[nblk];
 }
 
-template <bool Few>
 const void* sym_fn(int k) {
   switch (k) {
-    case 0: return reinterpret_cast<const void*>(k_small_sym<1, Few>);
-    case 1: return reinterpret_cast<const void*>(k_small_sym<2, Few>);
-    case 2: return reinterpret_cast<const void*>(k_small_sym<4, Few>);
-    case 3: return reinterpret_cast<const void*>(k_small_sym<8, Few>);
-    case 4: return reinterpret_cast<const void*>(k_small_sym<16, Few>);
-    default: return reinterpret_cast<const void*>(k_small_sym<32, Few>);
+    case 0: return reinterpret_cast<const void*>(k_small_sym<1, false>);
+    case 1: return reinterpret_cast<const void*>(k_small_sym<2, false>);
+    case 2: return reinterpret_cast<const void*>(k_small_sym<4, false>);
+    case 3: return reinterpret_cast<const void*>(k_small_sym<8, false>);
+    case 4: return reinterpret_cast<const void*>(k_small_sym<16, false>);
+    default: return reinterpret_cast<const void*>(k_small_sym<32, false>);
   }
 }
 
@@ -782,7 +794,7 @@ const void* num_fn(int k) {
 // Per device, once: the registers a thread of each kernel instance holds, and the numeric
 // kernels' dynamic shared memory limit raised to kNumSmemMax.
 struct SmallKernelInfo {
-  int sym_regs[2][kPerCount] = {}, num_regs[kPerCount] = {};
+  int sym_regs[kPerCount] = {}, few_regs[2] = {}, num_regs[kPerCount] = {};
   bool ready = false;
 };
 
@@ -796,16 +808,17 @@ const SmallKernelInfo& small_info() {
   if (static_cast<int>(g_small_info.size()) <= dev) g_small_info.resize(dev + 1);
   SmallKernelInfo& k = g_small_info[dev];
   if (!k.ready) {
-    for (int i = 0; i < kPerCount; ++i) {
+    auto regs = [](const void* f) {
       cudaFuncAttributes fa{};
-      for (int few = 0; few < 2; ++few)
-        k.sym_regs[few][i] = cudaFuncGetAttributes(&fa, few ? sym_fn<true>(i) : sym_fn<false>(i)) == cudaSuccess &&
-                                     fa.numRegs > 0
-                                 ? fa.numRegs
-                                 : 64;
-      k.num_regs[i] = cudaFuncGetAttributes(&fa, num_fn(i)) == cudaSuccess && fa.numRegs > 0 ? fa.numRegs : 64;
+      return cudaFuncGetAttributes(&fa, f) == cudaSuccess && fa.numRegs > 0 ? fa.numRegs : 64;
+    };
+    for (int i = 0; i < kPerCount; ++i) {
+      k.sym_regs[i] = regs(sym_fn(i));
+      k.num_regs[i] = regs(num_fn(i));
       cudaFuncSetAttribute(num_fn(i), cudaFuncAttributeMaxDynamicSharedMemorySize, kNumSmemMax);
     }
+    k.few_regs[0] = regs(reinterpret_cast<const void*>(k_small_sym<16, true>));
+    k.few_regs[1] = regs(reinterpret_cast<const void*>(k_small_sym<32, true>));
     cudaGetLastError();
     k.ready = true;
   }
@@ -847,14 +860,16 @@ bool small_path_fits(int64_t m, int64_t n) { return m <= kSmallMaxRows && n <= k
 
 SmallGrid small_sym_grid(const SmallCsr& A, const SmallCsr& B, int64_t width, int num_sms) {
   const int per = small_per(width);
-  // Short rows four at a time, sorted across the warp, where there are enough of them for every warp of
-  // the chip; with fewer the four take longer than four warps (1,000^2, 4 entries a row: 64 us against
-  // 60; 32,000^2: 98 against 108, 1 entry a row 85 against 102; a batch of 67,000 rows: 36 against 61 in
-  // the kernel). The averages are those of the whole product: a longer row takes the bitmap.
-  const bool few = A.rows >= int64_t(num_sms) * 64 && avg_row(A) <= kFewEntries &&
+  // Short rows four at a time, sorted across the warp, where the bitmap has more than 8,192 columns, which take
+  // a warp longer to clear and count than a sort, and where there are enough rows for every warp of the chip;
+  // with fewer the four take longer than four warps (1,000^2, 4 entries a row: 64 us against 60). The
+  // averages are those of the whole product: a longer row takes the bitmap. Kernel, us, of 65,000 rows of 9
+  // products, sorted 33, by bitmap of 32,000 columns 55, 16,000 35, 8,000 25, 100 24; of 30,000 rows 20 and 31, 24,
+  // 18, 18.
+  const bool few = per >= kFewPer && A.rows >= int64_t(num_sms) * 64 && avg_row(A) <= kFewEntries &&
                    avg_row(A) * avg_row(B) <= kFewProducts;
   const int G = few ? 4 : small_groups(avg_row(A), static_cast<size_t>(128) * per, kSymWarpBytes);
-  const int regs = small_info().sym_regs[few][per_index(per)];
+  const int regs = few ? small_info().few_regs[per > 16] : small_info().sym_regs[per_index(per)];
   const int64_t m = A.rows;
   const int64_t cap = int64_t(num_sms) * resident(regs, kSymWarps * 32, sym_smem(per, few ? 1 : G), 8);
   int64_t g = (m + int64_t(kSymWarps) * G - 1) / (int64_t(kSymWarps) * G);
