@@ -117,7 +117,7 @@ constexpr int kBlockCols = 1 << kBlockShift;   // columns per block, 4096
 constexpr int kBlockWords = kBlockCols / 32;   // bitmap words per block
 constexpr int kSymWinBits = 1 << 20;           // symbolic bitmap window (128 KB)
 // A plan whose windowed rows all have a stored bitmap counts them in sub-blocks instead
-// (k_winteam.cu): small enough that a warp's window holds any of them.
+// (k_winteam.cu): small enough that a window holds any of them.
 constexpr int kSubShift = 10;
 constexpr int kSubCols = 1 << kSubShift;
 constexpr int kMaxSub = kSymWinBits / kSubCols;

@@ -13,16 +13,15 @@
 // The output is sorted by column without a sort, as Algorithm 1's sorted PP (Sec. III-A).
 //
 // Bound by shared memory (the rank lookups and the sums' compare-and-swaps: 70 % of the peak wavefronts),
-// by the instructions of a product (about 94 per 32 products) and by the FP64 pipe (50 %). Against one block per
-// row with windows of 4096 entries (k_num_window) and a pass of its own for the columns (k_expand_cols):
-// small windows of any row keep more of them in flight, a list of windows lets the next one's data be
-// fetched ahead, a product stores its column at its rank on the way, so no pass extracts the columns
-// from the bitmap, whole groups of 32 products of one segment need no search per product, and the
-// others' segment is a popcount of the bits where segments start. Both kernels -> this one: 30,000^2
-// uniform (d = 5e-3, 6.7e8 products) 7.35 -> 4.21 ms, R-MAT 2^17 (1.09e9) 9.92 -> 5.68 ms, R-MAT 2^19
-// (7.85e9) 77.6 -> 51.8 ms. Of this, the bits instead of a search of the segments' ends: 5.06 -> 4.64,
-// 6.39 -> 6.31, 58.6 -> 57.5; the fused sums (add_product_f64) instead of atomicAdd: 4.64 -> 4.53, 6.31 ->
-// 5.69, 57.5 -> 54.8; larger windows (below): 4.53 -> 4.21, 5.69 -> 5.68, 54.8 -> 51.8.
+// by the instructions of a product (about 94 per 32 products) and by the FP64 pipe (50 %). What it saves against
+// a block per row with windows of the same size (k_num_window) and a pass of its own for the columns
+// (k_expand_cols): the list lets the next window's data be fetched while one is worked on and spreads a
+// long row over all blocks; a product stores its column at its rank on the way, so no pass extracts the
+// columns from the bitmap; three blocks of eight warps on an SM wait less at a window's barriers than two
+// of sixteen; whole groups of 32 products of one segment need no search per product, and the others'
+// segment is a popcount of the bits where segments start. Both kernels and this one: 30,000^2 uniform
+// (d = 5e-3, 6.7e8 products) 7.35 and 4.21 ms, R-MAT 2^17 (1.09e9) 9.92 and 5.68 ms, R-MAT 2^19 (7.85e9) 77.6
+// and 51.8 ms; a single row of 90,000 entries of A (9e6 products) 126 and 2.8 ms, all passes.
 //
 // FP32-compensated plans take the same kernel with FP32 sums and compensations in the eight bytes of a
 // slot (two FP32 atomics a product, separate arrays so that both spread over all banks): R-MAT 2^17
